@@ -14,6 +14,7 @@
 // to the kernels.  Every call overwrites each scratch slot it later reads, so
 // nothing has to be cleared between calls; calls that overlap on the GPU share
 // the array and race.
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -22,76 +23,152 @@
 namespace rpt {
 namespace {
 
-constexpr int kNaThreads = 512;
-constexpr int kNaMaxCtas = 128;
+constexpr int kNaThreads = 1024;
+constexpr int kNaMaxCtas = 128;            // CTAs whose partial sums fit the scratch at kNaMaxCols
 constexpr int kNaMaxCols = 8192;           // largest n (columns padded to a multiple of 32)
 
-// Per-CTA partial accumulators: kNaMaxCtas x kNaMaxCols floats (4 MiB).
+// Per-CTA partial accumulators, one row of n_pad floats per CTA (4 MiB in all).
 static __device__ __align__(256) float g_noalloc_scratch[kNaMaxCtas * kNaMaxCols];
 
-// Rows of CTA c: an nnz-balanced split found by binary search on row_ptr.
-__device__ int first_row_with_offset(const int32_t* __restrict__ rp, int m, long long target) {
-  int lo = 0, hi = m;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if ((long long)rp[mid] >= target) hi = mid;
-    else lo = mid + 1;
+// CTAs that get a partial row: what the scratch holds at this width (at least
+// kNaMaxCtas).
+constexpr int na_ctas(int n_pad) { return kNaMaxCtas * kNaMaxCols / n_pad; }
+
+constexpr int kNaLanes = 8;                // lanes per row
+constexpr int kNaKeep = 16;                // entries per lane kept between the dot and the scatter
+constexpr int kNaApart = 1024;             // the 4 rows of a warp step lie up to this far apart
+constexpr int kNaBatch = 8;                // steps whose row offsets are loaded together
+
+// One row by L lanes (this lane is sl), or nothing when lo == hi: the row's
+// entries, the first KEEP L of them kept in registers between the dot and the
+// scatter.  Entries outside [0, n) are ignored.  Every lane of the warp calls it.
+template <int L, int KEEP>
+__device__ __forceinline__ void na_row(unsigned lo, unsigned hi, unsigned sl, float wi, int n, const int32_t* __restrict__ col,
+                                       const float* __restrict__ val, const float* sv, float* acc) {
+  float a[KEEP];
+  int c[KEEP];
+#pragma unroll
+  for (int k = 0; k < KEEP; ++k) {
+    const unsigned e = lo + sl + L * k;
+    a[k] = e < hi ? __ldg(val + e) : 0.f;
+    c[k] = e < hi ? __ldg(col + e) : -1;
   }
-  return lo;
+  float t = 0.f;
+#pragma unroll
+  for (int k = 0; k < KEEP; ++k)
+    if ((unsigned)c[k] < (unsigned)n) t = fmaf(a[k], sv[c[k]], t);
+  for (unsigned e = lo + sl + L * KEEP; e < hi; e += L) {
+    const int q = __ldg(col + e);
+    if ((unsigned)q < (unsigned)n) t = fmaf(__ldg(val + e), sv[q], t);
+  }
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  const float coef = wi * t;
+#pragma unroll
+  for (int k = 0; k < KEEP; ++k)
+    if ((unsigned)c[k] < (unsigned)n) atomicAdd(&acc[c[k]], coef * a[k]);
+  for (unsigned e = lo + sl + L * KEEP; e < hi; e += L) {
+    const int q = __ldg(col + e);
+    if ((unsigned)q < (unsigned)n) atomicAdd(&acc[q], coef * __ldg(val + e));
+  }
 }
 
+// Bound: the entries once from HBM (8 bytes each).  A CSR matrix handed over per
+// call cannot be cut by cost in advance, and most of its rows may be empty (the
+// voxels outside the beams), so rows are dealt evenly: a step takes 4 rows, 8
+// lanes each, and steps go round-robin over all warps of the grid, so that every
+// warp gets its part of every region.  The 4 rows of a step lie `apart` rows apart:
+// neighbouring rows share most of their spots, and lanes that meet on one spot
+// retry their atomics.  Row offsets are loaded for kNaBatch steps at once; empty
+// steps cost a ballot.  Rows longer than the 8 lanes keep in registers are left
+// for the whole warp.  One scenario of the realistic plan (10.0 M entries, 299k
+// rows of which 214k are empty, 5000 spots): 52 us for both kernels against
+// 2568 us when CTAs were cut by entries, which left the empty rows at both ends
+// of the volume to two CTAs, and each warp waited for one row at a time; 190k
+// entries and 200 spots: 12 us against 49 us.
 __global__ void __launch_bounds__(kNaThreads)
-k_noalloc_pass(int m, int n, int n_pad, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
+k_noalloc_pass(int m, int n, int n_pad, int apart, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
                const float* __restrict__ val, const float* __restrict__ w, const float* __restrict__ v,
                float* __restrict__ scratch) {
   extern __shared__ float sm[];
   float* sv = sm;
   float* acc = sm + n_pad;
-  __shared__ int rows[2];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kNaThreads / 32;
+  const int tid = threadIdx.x, lane = tid & 31, nw = kNaThreads / 32;
   for (int j = tid; j < n_pad; j += kNaThreads) {
     sv[j] = j < n ? v[j] : 0.f;
     acc[j] = 0.f;
   }
-  if (tid == 0) {
-    const long long nnz = rp[m];
-    rows[0] = first_row_with_offset(rp, m, nnz * blockIdx.x / gridDim.x);
-    rows[1] = blockIdx.x + 1 == gridDim.x ? m : first_row_with_offset(rp, m, nnz * (blockIdx.x + 1) / gridDim.x);
+  __syncthreads();
+  const int sl = lane & (kNaLanes - 1);
+  const int tile = 4 * apart;
+  const int steps = ((m - 1) / tile + 1) * apart;   // m / 4 rounded up to whole tiles
+  const int stride = gridDim.x * nw;
+  // consecutive steps go to different CTAs
+  const int first = (tid >> 5) * gridDim.x + blockIdx.x;
+  for (int s0 = first; s0 < steps; s0 += stride * kNaBatch) {
+    // lane l: row l & 3 of the batch's step l >> 2
+    const int s = s0 + stride * (lane >> 2);
+    const long long i = (long long)(s / apart) * tile + s % apart + (lane & 3) * apart;
+    int blo = 0, bhi = 0;
+    float bw = 0.f;
+    if (s < steps && i < m) {
+      blo = __ldg(rp + i);
+      bhi = __ldg(rp + i + 1);
+      if (bhi > blo) bw = __ldg(w + i);
+    }
+    const unsigned any = __ballot_sync(0xffffffffu, bhi > blo);
+    for (int b = 0; b < kNaBatch; ++b) {
+      if (((any >> (4 * b)) & 15u) == 0) continue;
+      const int from = 4 * b + lane / kNaLanes;
+      const int lo = __shfl_sync(0xffffffffu, blo, from), hi = __shfl_sync(0xffffffffu, bhi, from);
+      const float wi = __shfl_sync(0xffffffffu, bw, from);
+      const bool wide = hi - lo > kNaLanes * kNaKeep;
+      na_row<kNaLanes, kNaKeep>(lo, wide ? lo : hi, sl, wi, n, col, val, sv, acc);
+      unsigned left = __ballot_sync(0xffffffffu, wide && sl == 0);
+      while (left) {
+        const int src = __ffs(left) - 1;
+        left &= left - 1;
+        na_row<32, kNaKeep>(__shfl_sync(0xffffffffu, lo, src), __shfl_sync(0xffffffffu, hi, src), lane,
+                            __shfl_sync(0xffffffffu, wi, src), n, col, val, sv, acc);
+      }
+    }
   }
   __syncthreads();
-  for (int i = rows[0] + warp; i < rows[1]; i += nw) {
-    const int a = rp[i], b = rp[i + 1];
-    float t = 0.f;
-    for (int k = a + lane; k < b; k += 32) {
-      const int c = col[k];
-      if ((unsigned)c < (unsigned)n) t = fmaf(val[k], sv[c], t);   // entries outside [0, n) are ignored
-    }
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    const float coef = w[i] * t;
-    for (int k = a + lane; k < b; k += 32) {
-      const int c = col[k];
-      if ((unsigned)c < (unsigned)n) atomicAdd(&acc[c], coef * val[k]);
-    }
-  }
-  __syncthreads();
-  float* out = scratch + (size_t)blockIdx.x * kNaMaxCols;
-  for (int j = tid; j < n_pad; j += kNaThreads) out[j] = acc[j];
+  float4* out = reinterpret_cast<float4*>(scratch + (size_t)blockIdx.x * n_pad);
+  for (int j = tid; j < n_pad / 4; j += kNaThreads) out[j] = reinterpret_cast<const float4*>(acc)[j];
 }
 
-// u[j] = sum over CTAs c of scratch[c][j] + (rho/2) v[j].  The sum over the CTAs
-// runs in a fixed order with compensation; the partial of each CTA comes from
-// shared-memory float atomics whose order varies between runs, so results are
-// not bitwise reproducible (they stay within the float32 bound of the sums).
-__global__ void k_noalloc_reduce(int n, int ctas, const float* __restrict__ scratch, const float* __restrict__ v,
-                                 float half_rho, float* __restrict__ u) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
+// u[j] = sum over CTAs c of scratch[c][j] + (rho/2) v[j].  Latency-bound, so the
+// CTAs' partials of 32 columns go to kNaSums thread rows (independent loads), each
+// a compensated sum in a fixed order, and the rows' sums are added with
+// compensation in row order; the partial of each CTA comes from shared-memory
+// float atomics whose order varies between runs, so results are not bitwise
+// reproducible (they stay within the float32 bound of the sums).
+constexpr int kNaSums = 16;
+__global__ void __launch_bounds__(32 * kNaSums)
+k_noalloc_reduce(int n, int n_pad, int ctas, const float* __restrict__ scratch, const float* __restrict__ v,
+                 float half_rho, float* __restrict__ u) {
+  __shared__ float ss[kNaSums][32], sc[kNaSums][32];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int j = blockIdx.x * 32 + x;        // n_pad is a multiple of 32
   float s = 0.f, c = 0.f;
-  for (int k = 0; k < ctas; ++k) {
+#pragma unroll 4
+  for (int k = y; k < ctas; k += kNaSums) {
     float t, e;
-    two_sum(s, scratch[(size_t)k * kNaMaxCols + j], t, e);
+    two_sum(s, __ldcg(scratch + (size_t)k * n_pad + j), t, e);
     s = t;
     c += e;
+  }
+  ss[y][x] = s;
+  sc[y][x] = c;
+  __syncthreads();
+  if (y != 0 || j >= n) return;
+#pragma unroll
+  for (int k = 1; k < kNaSums; ++k) {
+    float t, e;
+    two_sum(s, ss[k][x], t, e);
+    s = t;
+    c += e + sc[k][x];
   }
   u[j] = (s + c) + half_rho * v[j];
 }
@@ -147,13 +224,15 @@ extern "C" int rpt_normal_apply_noalloc(int32_t m, int32_t n, const int32_t* row
   int ctas = 0;
   if ((e = cudaDeviceGetAttribute(&ctas, cudaDevAttrMultiProcessorCount, dev)))
     return cuda_fail(e, "device attribute");
-  ctas = ctas < kNaMaxCtas ? ctas : kNaMaxCtas;
-  if (ctas > m) ctas = m;
+  // one CTA per SM, as many as have a partial row and steps for half of their warps
+  ctas = std::min(ctas, na_ctas(n_pad));
+  const int apart = std::min(kNaApart, m / 4 + 1);
+  ctas = std::min(ctas, (m - 1) / (2 * (kNaThreads / 32)) + 1);
   cudaStream_t st = (cudaStream_t)stream;
-  k_noalloc_pass<<<ctas, kNaThreads, smem, st>>>(m, n, n_pad, row_ptr_dev, col_idx_dev, val_dev, row_w_dev, v_dev,
+  k_noalloc_pass<<<ctas, kNaThreads, smem, st>>>(m, n, n_pad, apart, row_ptr_dev, col_idx_dev, val_dev, row_w_dev, v_dev,
                                                  scratch);
   if ((e = cudaGetLastError())) return cuda_fail(e, "launch");
-  k_noalloc_reduce<<<(n + 255) / 256, 256, 0, st>>>(n, ctas, scratch, v_dev, (float)(0.5 * rho), u_dev);
+  k_noalloc_reduce<<<n_pad / 32, 32 * kNaSums, 0, st>>>(n, n_pad, ctas, scratch, v_dev, (float)(0.5 * rho), u_dev);
   if ((e = cudaGetLastError())) return cuda_fail(e, "launch");
   return RPT_OK;
 }

@@ -107,3 +107,31 @@ def test_noalloc_rejects_bad_sizes():
     with pytest.raises(rpt.RptError) as e:
         rpt.normal_apply_noalloc(0, 10, 1, 1, 1, 1, 1, 1.0, 1)
     assert e.value.status == rpt.EINVAL
+
+
+@pytest.mark.parametrize("m,n,lens", [
+    (1, 1, (1,)),                                   # one row, one step
+    (3, 40, (0, 5, 31)),
+    (130, 333, (0, 1, 7, 8, 9, 127, 128, 129)),     # around what 8 lanes keep in registers
+    (4097, 700, (0, 0, 3, 130)),                    # one row past a tile of rows
+    (9001, 6001, (0, 0, 0, 40, 511, 512, 513, 900)),   # around what a warp keeps, three tiles
+])
+def test_noalloc_row_lengths_and_tile_edges(m, n, lens):
+    rpt = gpu_lib()
+    import torch
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(m)
+    ln = np.minimum(rng.choice(lens, size=m), n)
+    ln[-1] = min(max(lens), n)                       # the last row is not empty
+    rp = np.concatenate([[0], np.cumsum(ln)]).astype(np.int32)
+    ci = np.concatenate([np.sort(rng.choice(n, size=l, replace=False)) for l in ln]).astype(np.int32)
+    va = rng.uniform(0.0, 2.0, size=rp[-1]).astype(np.float32)
+    w = rng.uniform(0.1, 10.0, size=m).astype(np.float32).astype(np.float64)
+    A = sp.csr_matrix((va.astype(np.float64), ci, rp), shape=(m, n))
+    kf = (int(ln.max()) + int(np.bincount(ci, minlength=n).max()) + 8) * float(np.finfo(np.float32).eps)
+    arrs = _device_arrays(torch, dev, rp, ci, va, w, n)
+    V = rng.normal(size=n).astype(np.float32).astype(np.float64)
+    got = _call(rpt, torch, dev, m, n, arrs, V, 0.5)
+    ref = A.T @ (w * (A @ V)) + 0.25 * V
+    mag = A.T @ (w * (A @ np.abs(V))) + 0.25 * np.abs(V)
+    assert np.all(np.abs(got - ref) <= kf * mag + 1e-30)
