@@ -11,7 +11,8 @@
 //   BF16 (default): weights, activations and activation gradients enter the
 //     GEMMs as bfloat16 and the tensor cores accumulate in FP32 (gemm_bf16.cuh,
 //     mma.sync); the FP32 master weights take the Adam step and are rounded to
-//     the bfloat16 copy after it; biases, losses and gradients stay FP32.
+//     the bfloat16 copy after it; biases, losses and gradients stay FP32.  A pass
+//     is one launch per layer forward and one per layer backward.
 //   F32: the tiled shared-memory FP32 GEMM of gemm.cuh on the CUDA cores.
 // The network is small (under a million weights, batches of a few hundred rows),
 // so its GEMMs are latency- and launch-bound either way.
@@ -47,14 +48,21 @@ __global__ void k_bias_grad(int M, int N, const float* __restrict__ dH, float* _
   db[j] = s;
 }
 
-// dOut = 2 (Out - Y) / (M N); loss += sum (Out - Y)^2 / (M N)  (FP64 partial sums)
-__global__ void k_mse(int64_t n, const float* __restrict__ out, const float* __restrict__ y, float* __restrict__ d,
-                      double inv, double* __restrict__ loss) {
+// dOut = 2 (Out - Y) / (M N); loss += sum (Out - Y)^2 / (M N)  (FP64 partial sums);
+// db (or null): bfloat16 copy of dOut with leading dimension ldb
+__global__ void k_mse(int rows, int cols, const float* __restrict__ out, const float* __restrict__ y,
+                      float* __restrict__ d, __nv_bfloat16* __restrict__ db, int ldb, double inv,
+                      double* __restrict__ loss) {
   __shared__ double sh[32];
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int64_t n = (int64_t)rows * cols;
   double acc = 0.0;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
     const float e = out[k] - y[k];
-    d[k] = (float)(2.0 * inv) * e;
+    const float dk = (float)(2.0 * inv) * e;
+    d[k] = dk;
+    if (db) db[k / cols * ldb + k % cols] = __float2bfloat16_rn(dk);
     acc += (double)e * e;
   }
   double v[1] = {acc};
@@ -62,22 +70,114 @@ __global__ void k_mse(int64_t n, const float* __restrict__ out, const float* __r
   if (threadIdx.x == 0) atomicAdd(loss, v[0] * inv);
 }
 
-// Adam (Kingma & Ba, Algorithm 1) with bias correction folded into the step size.
-__global__ void k_adam(int64_t n, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, float lr_t, float b1, float b2, float eps, float wd) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+// Layers of a network, for kernels that run over all parameters (grid.y = layer).
+constexpr int kMaxLayers = 17;
+struct LayerTab {
+  int64_t woff[kMaxLayers], pboff[kMaxLayers];   // layer's parameters (W then b), its bfloat16 weights
+  int in[kMaxLayers], out[kMaxLayers], ld[kMaxLayers];
+};
+
+// Adam (Kingma & Ba, Algorithm 1) with bias correction folded into the step size;
+// pb (or null): the bfloat16 copy of the weights follows.
+__global__ void k_adam(const __grid_constant__ LayerTab T, float* __restrict__ p, const float* __restrict__ g,
+                       float* __restrict__ m, float* __restrict__ v, __nv_bfloat16* __restrict__ pb, float lr_t,
+                       float b1, float b2, float eps, float wd) {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int l = blockIdx.y, in = T.in[l], ld = T.ld[l];
+  const int64_t nw = (int64_t)in * T.out[l], n = nw + T.out[l];
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = T.woff[l] + q;
     const float gk = g[k] + wd * p[k];
     const float mk = b1 * m[k] + (1.f - b1) * gk;
     const float vk = b2 * v[k] + (1.f - b2) * gk * gk;
     m[k] = mk;
     v[k] = vk;
-    p[k] -= lr_t * mk / (sqrtf(vk) + eps);
+    const float pk = p[k] - lr_t * mk / (sqrtf(vk) + eps);
+    p[k] = pk;
+    if (pb && q < nw) pb[T.pboff[l] + q / in * ld + q % in] = __float2bfloat16_rn(pk);
   }
 }
 
-__global__ void k_to_bf16(int64_t n, const float* __restrict__ src, __nv_bfloat16* __restrict__ dst) {
+// The bfloat16 copy of the weights (grid.y = layer).
+__global__ void k_weights_bf16(const __grid_constant__ LayerTab T, const float* __restrict__ p,
+                               __nv_bfloat16* __restrict__ pb) {
+  const int l = blockIdx.y, in = T.in[l], ld = T.ld[l];
+  const int64_t nw = (int64_t)in * T.out[l];
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nw; q += (int64_t)gridDim.x * blockDim.x)
+    pb[T.pboff[l] + q / in * ld + q % in] = __float2bfloat16_rn(p[T.woff[l] + q]);
+}
+
+// dst [rows][ld] = bfloat16(src [rows][cols]); the padding stays as it is (zero).
+// zero (or null): set to 0 (the loss sum of the pass that follows).
+__global__ void k_to_bf16(int rows, int cols, int ld, const float* __restrict__ src,
+                          __nv_bfloat16* __restrict__ dst, double* zero) {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int64_t n = (int64_t)rows * cols;
+  if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0.0;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    dst[k] = __float2bfloat16_rn(src[k]);
+    dst[k / cols * ld + k % cols] = __float2bfloat16_rn(src[k]);
+}
+
+// Forward layer (BF16): C = act W^T + bias (+ ReLU), with its bfloat16 copy.
+template <int T>
+__global__ void __launch_bounds__(kTcThreads) k_layer_fwd(const __grid_constant__ TcGemm g) {
+  __shared__ __align__(16) __nv_bfloat16 sm[kTcStages<T> * kTcTile<T>];
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  tc_gemm_block<false, true, T>(g, blockIdx.x, sm);
+}
+
+// Backward of one layer (BF16) in one launch, since neither part waits for the
+// other: blocks [0, nx) the gradient of the layer's input, dx = dy W masked by
+// the ReLU below (nx = 0 for the first layer); [nx, nx + nw) the weights'
+// gradient dW = dy^T x; the rest the bias gradient, 128 columns each, summed
+// over the rows in order.
+template <int TX, int TW>
+__global__ void __launch_bounds__(kTcThreads)
+k_layer_bwd(const __grid_constant__ TcGemm gx, int nx, const __grid_constant__ TcGemm gw, int nw, int rows, int cols,
+            const float* __restrict__ dy, float* __restrict__ db) {
+  constexpr int kX = kTcStages<TX> * kTcTile<TX>, kW = kTcStages<TW> * kTcTile<TW>;
+  __shared__ __align__(16) __nv_bfloat16 sm[kX > kW ? kX : kW];
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int blk = blockIdx.x;
+  if (blk < nx) {
+    tc_gemm_block<false, false, TX>(gx, blk, sm);
+  } else if (blk < nx + nw) {
+    tc_gemm_block<true, false, TW>(gw, blk - nx, sm);
+  } else {
+    const int j = (blk - nx - nw) * kTcThreads + threadIdx.x;
+    if (j >= cols) return;
+    float s = 0.f;
+    int i = 0;
+    for (; i + 32 <= rows; i += 32) {       // loads of 32 rows in flight, added in order
+      float v[32];
+#pragma unroll
+      for (int u = 0; u < 32; ++u) v[u] = __ldcg(dy + (size_t)(i + u) * cols + j);
+#pragma unroll
+      for (int u = 0; u < 32; ++u) s += v[u];
+    }
+    for (; i < rows; ++i) s += __ldcg(dy + (size_t)i * cols + j);
+    db[j] = s;
+  }
+}
+
+// Launch that may begin while the stream's previous kernel drains (its threads
+// wait for that kernel's results before they read or write).
+template <typename... P, typename... A>
+void launch_next(cudaStream_t st, void (*fn)(P...), dim3 blocks, int threads, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = blocks;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, fn, P(args)...);
 }
 
 __global__ void k_gather_rows(int rows, int cols, const int* __restrict__ idx, const float* __restrict__ src,
@@ -99,8 +199,14 @@ struct Mlp {
   int64_t nparam = 0;
   float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
   int bf16 = 1;                       // compute form: 1 bfloat16 tensor cores, 0 FP32 CUDA cores
-  __nv_bfloat16* pb = nullptr;        // bfloat16 copy of p (the weights the BF16 GEMMs read)
-  std::vector<__nv_bfloat16*> actb, dactb;   // bfloat16 copies of act / dact
+  // bfloat16 operands of the BF16 GEMMs: the weights (layer l at pboff[l]) and
+  // the copies of act / dact, with leading dimensions padded to a multiple of 8
+  // (ldb[l] for width dims[l]) and zeros in the padding
+  __nv_bfloat16* pb = nullptr;
+  std::vector<int64_t> pboff;
+  std::vector<int> ldb;
+  std::vector<__nv_bfloat16*> actb, dactb;
+  int sm_count = 1;
   int cap = 0;                        // rows the activation buffers hold
   std::vector<float*> act;            // act[0] = input batch, act[l+1] = output of layer l
   std::vector<float*> dact;           // gradients w.r.t. act[l+1]
@@ -142,8 +248,11 @@ cudaError_t ensure_cap(Mlp* M, int rows) {
   for (int l = 0; l <= L && e == cudaSuccess; ++l) {
     e = cudaMalloc(&M->act[l], sizeof(float) * (size_t)rows * M->dims[l]);
     if (e == cudaSuccess) e = cudaMalloc(&M->dact[l], sizeof(float) * (size_t)rows * M->dims[l]);
-    if (e == cudaSuccess) e = cudaMalloc(&M->actb[l], sizeof(__nv_bfloat16) * (size_t)rows * M->dims[l]);
-    if (e == cudaSuccess) e = cudaMalloc(&M->dactb[l], sizeof(__nv_bfloat16) * (size_t)rows * M->dims[l]);
+    const size_t bb = sizeof(__nv_bfloat16) * (size_t)rows * M->ldb[l];
+    if (e == cudaSuccess) e = cudaMalloc(&M->actb[l], bb);
+    if (e == cudaSuccess) e = cudaMalloc(&M->dactb[l], bb);
+    if (e == cudaSuccess) e = cudaMemsetAsync(M->actb[l], 0, bb, M->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(M->dactb[l], 0, bb, M->stream);
   }
   if (e == cudaSuccess) e = cudaMalloc(&M->y, sizeof(float) * (size_t)rows * M->dims[L]);
   if (e == cudaSuccess) e = cudaMalloc(&M->idx, sizeof(int) * (size_t)rows);
@@ -153,51 +262,91 @@ cudaError_t ensure_cap(Mlp* M, int rows) {
 
 int blocks_for(int64_t n) { return (int)std::min<int64_t>(4096, std::max<int64_t>(1, (n + 255) / 256)); }
 
-// Forward pass of `rows` rows already in act[0].
+// Forward pass of `rows` rows already in act[0]; clears the loss sum.
 void forward(Mlp* M, int rows) {
   const int L = (int)M->dims.size() - 1;
-  if (M->bf16) {
-    const int64_t n0 = (int64_t)rows * M->dims[0];
-    k_to_bf16<<<blocks_for(n0), 256, 0, M->stream>>>(n0, M->act[0], M->actb[0]);
-  }
+  if (M->bf16)
+    launch_next(M->stream, k_to_bf16, blocks_for((int64_t)rows * M->dims[0]), 256, rows, M->dims[0], M->ldb[0],
+                (const float*)M->act[0], M->actb[0], M->loss);
+  else
+    cudaMemsetAsync(M->loss, 0, sizeof(double), M->stream);
   for (int l = 0; l < L; ++l) {
     const int in = M->dims[l], out = M->dims[l + 1];
-    if (M->bf16)
-      gemm_bf16<false, true>(M->stream, rows, out, in, M->actb[l], in, M->pb + M->woff[l], in, M->act[l + 1], out,
-                             M->actb[l + 1], M->p + M->boff[l], l + 1 < L);
-    else
+    if (M->bf16) {
+      TcGemm g{};
+      g.M = rows;
+      g.N = out;
+      g.K = in;
+      g.A = M->actb[l];
+      g.lda = M->ldb[l];
+      g.B = M->pb + M->pboff[l];
+      g.ldb = M->ldb[l];
+      g.C = M->act[l + 1];
+      g.ldc = out;
+      g.Cb = l + 1 < L ? M->actb[l + 1] : nullptr;
+      g.ldcb = M->ldb[l + 1];
+      g.bias = M->p + M->boff[l];
+      g.relu = l + 1 < L;
+      if (tc_large(g, M->sm_count)) launch_next(M->stream, k_layer_fwd<64>, tc_tiles<64>(g), kTcThreads, g);
+      else launch_next(M->stream, k_layer_fwd<32>, tc_tiles<32>(g), kTcThreads, g);
+    } else {
       gemm<false, true>(M->stream, rows, out, in, M->act[l], in, M->p + M->woff[l], in, M->act[l + 1], out,
                         M->p + M->boff[l], l + 1 < L);
+    }
   }
 }
 
-// Loss and gradient of the batch (targets in M->y) into M->g; returns through M->loss.
+// Loss and gradient of the batch (targets in M->y) into M->g, after forward();
+// the loss through M->loss.
 void backward(Mlp* M, int rows) {
   const int L = (int)M->dims.size() - 1;
   const int nout = M->dims[L];
   const int64_t n = (int64_t)rows * nout;
-  cudaMemsetAsync(M->loss, 0, sizeof(double), M->stream);
-  k_mse<<<blocks_for(n), 256, 0, M->stream>>>(n, M->act[L], M->y, M->dact[L], 1.0 / (double)n, M->loss);
+  launch_next(M->stream, k_mse, blocks_for(n), 256, rows, nout, (const float*)M->act[L], (const float*)M->y,
+              M->dact[L], M->bf16 ? M->dactb[L] : nullptr, M->ldb[L], 1.0 / (double)n, M->loss);
   for (int l = L - 1; l >= 0; --l) {
     const int in = M->dims[l], out = M->dims[l + 1];
-    if (l + 1 < L) {
-      const int64_t k = (int64_t)rows * out;
-      k_relu_bwd<<<blocks_for(k), 256, 0, M->stream>>>(k, M->act[l + 1], M->dact[l + 1]);
-    }
-    k_bias_grad<<<(out + 255) / 256, 256, 0, M->stream>>>(rows, out, M->dact[l + 1], M->g + M->boff[l]);
     if (M->bf16) {
-      const int64_t k = (int64_t)rows * out;
-      k_to_bf16<<<blocks_for(k), 256, 0, M->stream>>>(k, M->dact[l + 1], M->dactb[l + 1]);
-      // dW_l = dAct_{l+1}^T act_l   ([out][rows] x [rows][in])
-      gemm_bf16<true, false>(M->stream, out, in, rows, M->dactb[l + 1], out, M->actb[l], in, M->g + M->woff[l],
-                             in);
-      // dAct_l = dAct_{l+1} W_l   ([rows][out] x [out][in]); not needed for the input
-      if (l > 0)
-        gemm_bf16<false, false>(M->stream, rows, in, out, M->dactb[l + 1], out, M->pb + M->woff[l], in,
-                                M->dact[l], in);
+      TcGemm gx{}, gw{};
+      gx.M = rows;              // dx = dy W, masked by the ReLU below; not needed for the input
+      gx.N = in;
+      gx.K = out;
+      gx.A = M->dactb[l + 1];
+      gx.lda = M->ldb[l + 1];
+      gx.B = M->pb + M->pboff[l];
+      gx.ldb = M->ldb[l];
+      gx.C = M->dact[l];
+      gx.ldc = in;
+      gx.Cb = M->dactb[l];
+      gx.ldcb = M->ldb[l];
+      gx.mask = M->act[l];
+      gw.M = out;               // dW = dy^T x
+      gw.N = in;
+      gw.K = rows;
+      gw.A = M->dactb[l + 1];
+      gw.lda = M->ldb[l + 1];
+      gw.B = M->actb[l];
+      gw.ldb = M->ldb[l];
+      gw.C = M->g + M->woff[l];
+      gw.ldc = in;
+      const bool lx = tc_large(gx, M->sm_count), lw = tc_large(gw, M->sm_count);
+      const int nx = l == 0 ? 0 : lx ? tc_tiles<64>(gx) : tc_tiles<32>(gx);
+      const int nw = lw ? tc_tiles<64>(gw) : tc_tiles<32>(gw);
+      const int blocks = nx + nw + (out + kTcThreads - 1) / kTcThreads;
+      auto* fn = lx ? (lw ? k_layer_bwd<64, 64> : k_layer_bwd<64, 32>)
+                    : (lw ? k_layer_bwd<32, 64> : k_layer_bwd<32, 32>);
+      launch_next(M->stream, fn, blocks, kTcThreads, gx, nx, gw, nw, rows, out, (const float*)M->dact[l + 1],
+                  M->g + M->boff[l]);
     } else {
+      if (l + 1 < L) {
+        const int64_t k = (int64_t)rows * out;
+        k_relu_bwd<<<blocks_for(k), 256, 0, M->stream>>>(k, M->act[l + 1], M->dact[l + 1]);
+      }
+      k_bias_grad<<<(out + 255) / 256, 256, 0, M->stream>>>(rows, out, M->dact[l + 1], M->g + M->boff[l]);
+      // dW_l = dAct_{l+1}^T act_l   ([out][rows] x [rows][in])
       gemm<true, false>(M->stream, out, in, rows, M->dact[l + 1], out, M->act[l], in, M->g + M->woff[l], in,
                         nullptr, false);
+      // dAct_l = dAct_{l+1} W_l   ([rows][out] x [out][in]); not needed for the input
       if (l > 0)
         gemm<false, false>(M->stream, rows, in, out, M->dact[l + 1], out, M->p + M->woff[l], in, M->dact[l], in,
                            nullptr, false);
@@ -207,9 +356,28 @@ void backward(Mlp* M, int rows) {
 
 int check(cudaError_t e, const char* what) { return e == cudaSuccess ? RPT_OK : cuda_fail(e, what); }
 
-// the bfloat16 copy of the weights, after every change of the FP32 ones
+LayerTab layers(const Mlp* M) {
+  LayerTab T{};
+  for (size_t l = 0; l + 1 < M->dims.size(); ++l) {
+    T.woff[l] = M->woff[l];
+    T.pboff[l] = M->pboff[l];
+    T.in[l] = M->dims[l];
+    T.out[l] = M->dims[l + 1];
+    T.ld[l] = M->ldb[l];
+  }
+  return T;
+}
+
+// grid of a kernel over all parameters: the widest layer's blocks, one row per layer
+dim3 layer_grid(const Mlp* M) {
+  int64_t n = 0;
+  for (size_t l = 0; l + 1 < M->dims.size(); ++l) n = std::max(n, (int64_t)(M->dims[l] + 1) * M->dims[l + 1]);
+  return dim3((unsigned)blocks_for(n), (unsigned)(M->dims.size() - 1));
+}
+
+// the bfloat16 copy of the weights, after the FP32 ones were set
 cudaError_t refresh_bf16(Mlp* M) {
-  k_to_bf16<<<blocks_for(M->nparam), 256, 0, M->stream>>>(M->nparam, M->p, M->pb);
+  k_weights_bf16<<<layer_grid(M), 256, 0, M->stream>>>(layers(M), M->p, M->pb);
   return cudaGetLastError();
 }
 
@@ -261,6 +429,12 @@ int rpt_mlp_create(int32_t n_in, int32_t n_hidden, int32_t n_hidden_layers, int3
     M->boff.push_back(M->nparam);
     M->nparam += M->dims[l + 1];
   }
+  int64_t npb = 0;
+  for (int l = 0; l <= L; ++l) {
+    M->ldb.push_back((M->dims[l] + 7) / 8 * 8);
+    M->pboff.push_back(npb);
+    if (l < L) npb += (int64_t)M->dims[l + 1] * M->ldb[l];
+  }
   // Glorot-uniform weights, zero biases, from a seeded host generator
   std::vector<float> h((size_t)M->nparam, 0.f);
   std::mt19937_64 gen(seed);
@@ -275,7 +449,9 @@ int rpt_mlp_create(int32_t n_in, int32_t n_hidden, int32_t n_hidden_layers, int3
   if (e == cudaSuccess) e = cudaMalloc(&M->m, bytes);
   if (e == cudaSuccess) e = cudaMalloc(&M->v, bytes);
   if (e == cudaSuccess) e = cudaMalloc(&M->loss, sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&M->pb, sizeof(__nv_bfloat16) * (size_t)M->nparam);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&M->sm_count, cudaDevAttrMultiProcessorCount, device);
+  if (e == cudaSuccess) e = cudaMalloc(&M->pb, sizeof(__nv_bfloat16) * (size_t)npb);
+  if (e == cudaSuccess) e = cudaMemsetAsync(M->pb, 0, sizeof(__nv_bfloat16) * (size_t)npb, M->stream);
   if (e == cudaSuccess) e = cudaMemcpy(M->p, h.data(), bytes, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = refresh_bf16(M);
   if (e == cudaSuccess) e = cudaStreamSynchronize(M->stream);
@@ -456,10 +632,9 @@ int rpt_mlp_train(rpt_mlp* mlp, const float* X, const float* Y, int32_t n, const
       const double bc1 = 1.0 - std::pow(tp->beta1, (double)M->step);
       const double bc2 = 1.0 - std::pow(tp->beta2, (double)M->step);
       const float lr_t = (float)(tp->lr * std::sqrt(bc2) / bc1);
-      k_adam<<<blocks_for(M->nparam), 256, 0, M->stream>>>(M->nparam, M->p, M->g, M->m, M->v, lr_t, b1, b2,
-                                                           (float)tp->eps, (float)tp->weight_decay);
+      launch_next(M->stream, k_adam, layer_grid(M), 256, layers(M), M->p, (const float*)M->g, M->m, M->v,
+                  M->bf16 ? M->pb : nullptr, lr_t, b1, b2, (float)tp->eps, (float)tp->weight_decay);
       e = cudaGetLastError();
-      if (e == cudaSuccess && M->bf16) e = refresh_bf16(M);
     }
     // stream ordering keeps the host-side permutation valid: wait before the next shuffle
     if (e == cudaSuccess) e = cudaStreamSynchronize(M->stream);

@@ -71,6 +71,33 @@ def test_bf16_tensor_core_gradient_matches_oracle(rpt, dims, rows):
     print(f"bfloat16 form vs exact float64 network, worst weight-gradient tensor: {worst:.2e}")
 
 
+@pytest.mark.parametrize("dims,rows", [
+    ([4, 9], 1),                  # one layer, one row
+    ([9, 33, 31], 65),            # one past a tile in rows, leading dimensions that need padding
+    ([9, 40, 1300], 500),         # 64 x 64 tiles forward only
+    ([3, 1301, 45], 500),         # 64 x 64 tiles for the input gradient, 32 x 32 for the weights
+    ([5, 700, 900], 3),           # and the other way round
+])
+def test_bf16_tile_choices_match_oracle(rpt, dims, rows):
+    """Every tile size of the BF16 form's products and its ragged edges, by the
+    rule of test_bf16_tensor_core_gradient_matches_oracle (1e-3 in norm)."""
+    from oracle.mlp import unpack, bf16_operand
+    rng = np.random.default_rng(8)
+    X = rng.normal(size=(rows, dims[0])).astype(np.float32)
+    Y = rng.normal(size=(rows, dims[-1])).astype(np.float32)
+    with rpt.Mlp(dims[0], dims[1] if len(dims) > 2 else 1, len(dims) - 2, dims[-1], seed=9) as net:
+        p = net.get_params().astype(np.float64)
+        loss, g = net.loss_grad(X, Y)
+        out = net.predict(X)
+    ref_out = forward(p, dims, X, bf16_operand)[-1]
+    assert np.linalg.norm(out - ref_out) <= 1e-3 * np.linalg.norm(ref_out)
+    ref_loss, ref_g = loss_grad(p, dims, X, Y, bf16_operand)
+    assert loss == pytest.approx(ref_loss, rel=1e-3)
+    for (W, b), (Wr, br) in zip(unpack(g, dims), unpack(ref_g, dims)):
+        assert np.linalg.norm(W - Wr) <= 1e-3 * np.linalg.norm(Wr)
+        assert np.linalg.norm(b - br) <= 1e-3 * np.linalg.norm(br)
+
+
 def test_set_params_round_trip_and_training_reduces_loss(rpt):
     rng = np.random.default_rng(4)
     X = rng.uniform(-1, 1, size=(512, 4)).astype(np.float32)
