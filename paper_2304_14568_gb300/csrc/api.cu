@@ -181,6 +181,17 @@ void free_plan(Plan* P) {
 
 using namespace layout;   // lanes per row, row lists, bank balance, chunks (layout.h)
 
+// Pass with private accumulators: consumer warps, bytes that its ring has at
+// least, units cut per CTA.  Twelve warps beat ten (0.166 against 0.187 ms on the
+// realistic plan) and leave 128 registers a thread.  Fewer accumulators make room
+// for the ring but more warps wait for a turn: with a ring of 72 KB (six
+// accumulators) the realistic plan took 0.213 ms against 0.166 with 128 KB (four);
+// twelve against six accumulators cost 0.066 against 0.057 ms at 2000 spots, three
+// against two gain 0.066 against 0.071 at 7000.
+constexpr int kPrivWarps = 12;
+constexpr size_t kPrivRing = 98304;
+constexpr int kUnitsPerCta = 64;
+
 // One bulk-copy ring configuration and its chunk lists.
 struct RingCfg {
   int cmax = 0, rmax = 0, stages = 0;
@@ -462,6 +473,9 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
   bool use_tma = false, use_stream = false;
   int ctas = 0;
   std::vector<RingCfg> ring_cfgs;   // ring configurations that fit (all of them when autotuning)
+  // bundled layout, private accumulators: item classes, units
+  std::vector<ItemClasses> icls;
+  std::vector<int> ubeg, uoff(N + 1, 0);
   // ---- bundled layout (path 4) ----
   if (want_path == 4 || want_path == 0) {
     std::vector<int3> cands = ring_override(opts, 3072, 192, 2);
@@ -747,6 +761,28 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
     dp.grid = P->sm_count * ctas;
     dp.nblocks = dp.grid * N;
     dp.slot_cap = dp.grid;
+    // private accumulators, unless the caller set the ring's geometry; at least two
+    // beside a ring of kPrivRing bytes (about 10,500 spots), three with fixed-point
+    // sums (4,600 spots), which hold their turn longer: at 5000 spots two took 0.294
+    // ms against the ring's 0.267.  Batched plans keep the ring: with three CTAs or so
+    // to a unit the float sums are grouped so differently that the iterates of a
+    // batched solve move by more than the ring's spread from run to run.
+    if (G == 1 && !want_thr && ring_override(opts, 1, 1, 2).empty()) {
+      int widest = 0;
+      cut_units(R, N, (int64_t)dp.grid * kUnitsPerCta, 4 * bv + bi, &icls, &ubeg, &uoff, &widest);
+      // the ring's bytes an item takes at most: columns, 16-byte alignment of both
+      // copies' ends, four records and a terminator's first 16 bytes
+      const size_t item = (size_t)widest * (4 * bv + bi) + 64 + 4 * 64 + 16;
+      const size_t room = (size_t)smem_optin - 1024;
+      for (int a : {6, 4, 3, 2}) {     // accumulators of the 12 consumer warps
+        const size_t fixed = priv_fixed_bytes(n_pad, a, exact);
+        if (fixed + std::max(kPrivRing, 2 * item) > room || (exact && a < 3)) continue;
+        dp.priv = kPrivWarps;
+        dp.priv_acc = a;
+        dp.ring_bytes = (int)std::min((room - fixed) & ~(size_t)127, (size_t)1 << 18);
+        break;
+      }
+    }
   }
   // slot lists: static for the register path (block b of scenario s), written
   // by the kernel for the bulk-copy path
@@ -774,6 +810,12 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
   for (const RingCfg& rc : ring_cfgs) chunk_cap = std::max(chunk_cap, rc.chunks.size());
   ChunkDesc* d_chunks = dyn ? A.get<ChunkDesc>(chunk_cap) : nullptr;
   int* d_scen_chunk = dyn ? A.get<int>(N + 1) : nullptr;
+  std::vector<int4> cls_h(dp.priv ? N : 0);
+  for (size_t s = 0; s < cls_h.size(); ++s)
+    cls_h[s] = make_int4(icls[s].n32, icls[s].n16, icls[s].n8, icls[s].items());
+  int4* d_cls = A.get<int4>(cls_h.size());
+  int* d_ubeg = A.get<int>(ubeg.size());
+  int* d_uoff = A.get<int>(N + 1);
   int* d_qnext = dyn ? A.get<int>(N) : nullptr;
   unsigned char* d_visited = dyn ? A.get<unsigned char>((size_t)N * dp.grid) : nullptr;
   int* d_slot_count = A.get<int>(N);
@@ -865,6 +907,9 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
     RPT_CP(d_chunks, chunks.data(), chunks.size() * sizeof(ChunkDesc));
     RPT_CP(d_scen_chunk, scen_chunk.data(), (N + 1) * sizeof(int));
   }
+  RPT_CP(d_cls, cls_h.data(), cls_h.size() * sizeof(int4));
+  RPT_CP(d_ubeg, ubeg.data(), ubeg.size() * sizeof(int));
+  RPT_CP(d_uoff, uoff.data(), (N + 1) * sizeof(int));
   RPT_CP(d_slot_count, slot_count.data(), N * sizeof(int));
   RPT_CP(d_slot_list, slot_list.data(), slot_list.size() * sizeof(int));
   RPT_CP(P->lb, lb.data(), lb.size() * sizeof(double));
@@ -892,6 +937,9 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
   dp.rec_base = d_recbase;
   dp.chunks = d_chunks;
   dp.scen_chunk = d_scen_chunk;
+  dp.cls = d_cls;
+  dp.ubeg = d_ubeg;
+  dp.uoff = d_uoff;
   dp.qnext = d_qnext;
   dp.visited = d_visited;
   dp.slot_count = d_slot_count;
@@ -1046,6 +1094,7 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
   S.autotune_seconds = 0.0;
   // ---- autotuning: time every fitting ring configuration on this plan, keep the fastest ----
   if ((use_tma || bundled) && ring_cfgs.size() > 1) {
+    const int priv = dp.priv;
     std::vector<double> ms(ring_cfgs.size(), 1e30);
     auto apply = [&](const RingCfg& rc) -> cudaError_t {
       cudaError_t ee = cudaMemcpyAsync(d_chunks, rc.chunks.data(), rc.chunks.size() * sizeof(ChunkDesc),
@@ -1056,6 +1105,7 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
       P->dp.cmax = rc.cmax;
       P->dp.rmax = rc.rmax;
       P->dp.stages = rc.stages;
+      P->dp.priv = 0;
       if (bundled) P->dp.ring_threads = rc.thr;
       if (ee == cudaSuccess) ee = rowpass_prepare(P->dp);
       return ee;
@@ -1091,10 +1141,24 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
         free_plan(P);
         return rc;
       }
+    double priv_ms = 1e30;
+    for (int k = 0; k < 2 && priv; ++k) {   // the pass with private accumulators against them
+      P->dp.priv = priv;
+      double t = 0.0, by = 0.0;
+      if (int rc = profile_row_pass(P, kNormal, 10, &t, &by)) {
+        free_plan(P);
+        return rc;
+      }
+      priv_ms = std::min(priv_ms, t);
+    }
     const size_t best = (size_t)(std::min_element(ms.begin(), ms.end()) - ms.begin());
     if ((e = apply(ring_cfgs[best]))) {
       free_plan(P);
       return cuda_fail(e, "autotune");
+    }
+    if (priv_ms <= ms[best]) {
+      P->dp.priv = priv;
+      ms[best] = priv_ms;
     }
     S.chunk_entries = ring_cfgs[best].cmax;
     S.chunk_rows = ring_cfgs[best].rmax;

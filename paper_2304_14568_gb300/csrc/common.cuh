@@ -89,6 +89,12 @@ struct DevPlan {
   int acc64;                          // 1: partial slots are int64 fixed point (path 3 with exact sums;
                                       //    0 on path 3: float32 shared atomics, like paths 0-2)
   int* fexp;                          // [N] scale exponent of the last scatter pass per scenario
+  int priv;                           // path 3: consumer warps of the pass with private accumulators
+                                      // (rowpriv.cu), 0: the ring with atomics; its accumulators (a divisor
+  int priv_acc, ring_bytes;           // of priv) and its ring's bytes; per scenario {bundles of 32 lanes, of 16, of 8, items}, the first unit
+  const int4* cls;                    // (scenario-major, [N+1]) and each unit's first item
+  const int* uoff;
+  const int* ubeg;
   const double* kbound;               // [2N] max_c sum_i c_s w_i |a_ic| ||a_i||_1 and max_c sum_i c_s w_i |a_ic| p_i
 };
 
@@ -164,6 +170,11 @@ size_t tma_smem_bytes(int n_pad, int cmax, int rmax, int stages, int value_bytes
                       bool scatter, bool bundled = false, bool fixed = false);
 size_t stream_smem_bytes(int n_pad, int rmax, bool scatter);
 void* stream_rowpass_kernel(const DevPlan& P, int mode);   // rowstream.cu
+// rowpriv.cu: every mode of a path-3 plan whose P.priv > 0
+inline bool use_priv(const DevPlan& P) { return P.path == 3 && P.priv > 0; }
+void* priv_rowpass_kernel(const DevPlan& P, int mode);
+int priv_threads(int warps);            // CTA size with that many consumer warps
+size_t priv_fixed_bytes(int n_pad, int accs, bool fixed);   // shared memory before its ring
 // Bundled layout, at plan creation: kbound[2s], kbound[2s+1] of every scenario
 // (DevPlan::kbound) from the stored values; kc, pc: scratch [n_pad] doubles.
 cudaError_t bundle_bounds(const DevPlan& P, double* kc, double* pc, double* kbound, cudaStream_t st);

@@ -426,5 +426,87 @@ inline void build_bundles_all(const std::vector<std::vector<BundleInRow>>& rows,
   });
 }
 
+// ---- work of the pass with private accumulators ---------------------------
+// A scenario's sorted bundles form items of 32 lanes: one bundle of 32 lanes, up
+// to two of 16 or up to four of 8 (bundle_lanes), in that order as the bundles
+// are sorted by decreasing width.
+struct ItemClasses {
+  int n32 = 0, n16 = 0, n8 = 0;   // bundles of each class
+  int items() const { return n32 + (n16 + 1) / 2 + (n8 + 3) / 4; }
+};
+
+// off: the scenario's bundle records' offsets (.x) of nb bundles and the terminator.
+inline ItemClasses item_classes(const int4* rec, int nb) {
+  ItemClasses c;
+  for (int q = 0; q < nb; ++q) {
+    const int g = bundle_lanes(rec[q + 1].x - rec[q].x);
+    ++(g == 32 ? c.n32 : g == 16 ? c.n16 : c.n8);
+  }
+  return c;
+}
+
+// Bundles [q, q + cnt) of item it.
+inline void item_range(const ItemClasses& c, int it, int* q, int* cnt) {
+  const int n16 = (c.n16 + 1) / 2;
+  if (it < c.n32) {
+    *q = it;
+    *cnt = 1;
+  } else if ((it -= c.n32) < n16) {
+    *q = c.n32 + 2 * it;
+    *cnt = std::min(2, c.n16 - 2 * it);
+  } else {
+    it -= n16;
+    *q = c.n32 + c.n16 + 4 * it;
+    *cnt = std::min(4, c.n8 - 4 * it);
+  }
+}
+
+// Units: every scenario's items cut into runs of about equal cost, so that a CTA
+// can take an equal share of any set of scenarios.  An item costs the bytes of its
+// block columns (col_bytes each) plus those that could be read in the time of its
+// reduction, coefficients and turns, measured per class.  Unit k of a scenario
+// begins with the first item that has at least k targets of cost before it (target
+// = total cost / parts), so any run of units is off by one item at most; a unit
+// inside a costly item is empty.  ubeg: each unit's first item, scenario-major;
+// uoff [N+1]; cls [N]; widest: block columns of the widest item.
+constexpr int kItemCost32 = 3000, kItemCost16 = 3700, kItemCost8 = 5300;
+constexpr int kWideKeep = 12;      // block columns per lane that 32 lanes keep in registers (rowpriv.cu)
+constexpr int kTailCost = 26;      // each block column beyond them, read twice
+
+inline void cut_units(const RowLists& R, int N, int64_t parts, int col_bytes, std::vector<ItemClasses>* cls,
+                      std::vector<int>* ubeg, std::vector<int>* uoff, int* widest) {
+  cls->assign(N, ItemClasses());
+  int64_t total = 0;
+  *widest = 0;
+  auto cost = [&](int s, int it) {
+    int q, cnt;
+    item_range((*cls)[s], it, &q, &cnt);
+    const int4* r = &R.rec[R.rec_base[s]];
+    const int w = r[q + cnt].x - r[q].x;
+    *widest = std::max(*widest, w);
+    const ItemClasses& c = (*cls)[s];
+    return (int64_t)w * col_bytes + (int64_t)std::max(0, it < c.n32 ? w - 32 * kWideKeep : 0) * kTailCost +
+           (it < c.n32 ? kItemCost32 : it < c.n32 + (c.n16 + 1) / 2 ? kItemCost16 : kItemCost8);
+  };
+  for (int s = 0; s < N; ++s) {
+    (*cls)[s] = item_classes(&R.rec[R.rec_base[s]], R.nrows[s]);
+    for (int it = 0; it < (*cls)[s].items(); ++it) total += cost(s, it);
+  }
+  const int64_t target = std::max<int64_t>(1, total / std::max<int64_t>(1, parts));
+  ubeg->clear();
+  uoff->assign(N + 1, 0);
+  for (int s = 0; s < N; ++s) {
+    (*uoff)[s] = (int)ubeg->size();
+    int64_t cum = 0, next = 0;   // cost before the item, cost at which the next unit begins
+    for (int it = 0; it < (*cls)[s].items(); ++it) {
+      for (; cum >= next; next += target) ubeg->push_back(it);
+      cum += cost(s, it);
+    }
+    // the units that begin inside the last item
+    for (; next < cum; next += target) ubeg->push_back((*cls)[s].items());
+  }
+  (*uoff)[N] = (int)ubeg->size();
+}
+
 }  // namespace layout
 }  // namespace rpt

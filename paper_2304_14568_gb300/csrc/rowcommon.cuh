@@ -87,6 +87,89 @@ template <> __device__ __forceinline__ void quad_c<false, uint16_t>(const uint16
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
+
+// ---------------------------------------------------------------------------
+// mbarrier / bulk-copy primitives (inline PTX)
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// try_wait with a suspend-time hint: a waiting thread sleeps until the phase
+// completes or about 0.1 ms pass, instead of spinning and taking issue slots
+// from the warps that work.
+constexpr uint32_t kSuspendHintNs = 100000;
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(kSuspendHintNs)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// Bounded wait for the phase with the given parity to complete: gives up after
+// one second of device time (try_wait itself may suspend the thread for a while,
+// so the bound is on time, not on the number of tries).
+constexpr unsigned long long kWaitLimitNs = 1000000000ull;
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const unsigned long long t0 = global_ns();
+  for (;;) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if (global_ns() - t0 > kWaitLimitNs) return false;
+  }
+}
+// Bulk copy global -> shared; completion is counted in bytes on `bar`.
+// dst, src 16-byte aligned; bytes a multiple of 16.
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void named_sync(int id, int count) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// Round y (a float32 of magnitude below 2^62) to the nearest integer, halves away
+// from zero, with integer operations on its bits: y = m 2^e with m the 24-bit
+// significand, so the result is m << e, or (m + 2^(-e-1)) >> -e when e < 0.  (A
+// float-to-64-bit-integer conversion instruction runs on the FP64 pipe, which is
+// narrow on this GPU.)  Zero and subnormal inputs give 0.
+__device__ __forceinline__ long long fixed_round(float y) {
+  const unsigned b = __float_as_uint(y);
+  const int e = (int)((b >> 23) & 0xffu) - 150;
+  if (e < -24) return 0;                              // |y| < 0.5
+  const long long m = (long long)((b & 0x7fffffu) | 0x800000u);
+  const long long q = e >= 0 ? (m << e) : ((m + (1ll << (-e - 1))) >> (-e));
+  return (b >> 31) ? -q : q;
+}
+
+// Scale exponent F of the fixed-point accumulation: 2^F * bound <= 2^60, so
+// that no sum of up to 2^2 times the bound (float32 rounding of the products
+// included) can overflow 63 bits; kFexpNaN marks a non-finite vector.
+__device__ __forceinline__ int fixed_exp(float vmax, double k, double pterm) {
+  if (!isfinite(vmax)) return kFexpNaN;
+  const double bound = k * (double)vmax + pterm;
+  if (!(bound > 0.0)) return 0;
+  int e;
+  frexp(bound, &e);                              // bound < 2^e
+  return max(-126, min(126, 60 - e));
+}
+
 // Stage v_s (scaled by the column scales of quantised values) into sv, zero acc.
 template <bool kScatter>
 __device__ __forceinline__ void stage_vector(const DevPlan& P, const float* __restrict__ vin, int v_stride,

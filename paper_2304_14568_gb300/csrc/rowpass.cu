@@ -36,62 +36,6 @@ namespace rpt {
 namespace {
 
 
-// ---------------------------------------------------------------------------
-// mbarrier / bulk-copy primitives (inline PTX)
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// try_wait with a suspend-time hint: a waiting thread sleeps until the phase
-// completes or about 0.1 ms pass, instead of spinning and taking issue slots
-// from the warps that work.
-constexpr uint32_t kSuspendHintNs = 100000;
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(kSuspendHintNs)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// Bounded wait for the phase with the given parity to complete: gives up after
-// one second of device time (try_wait itself may suspend the thread for a while,
-// so the bound is on time, not on the number of tries).
-constexpr unsigned long long kWaitLimitNs = 1000000000ull;
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  for (;;) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (global_ns() - t0 > kWaitLimitNs) return false;
-  }
-}
-// Bulk copy global -> shared; completion is counted in bytes on `bar`.
-// dst, src 16-byte aligned; bytes a multiple of 16.
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-__device__ __forceinline__ void named_sync(int id, int count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
 // One group of G lanes processes one row (G in {1, 2, ..., 32}); a warp covers
 // 32/G rows at once.  Lane sl of the group takes entries sl, sl + G, ... so that
 // the lanes of one instruction touch consecutive entries (consecutive spot
@@ -150,20 +94,6 @@ __device__ __forceinline__ void process_rows(const int4* __restrict__ rec, int r
       if (a != 0.f) atomicAdd(&acc[(int)col[idx]], coef * a);
     }
   }
-}
-
-// Round y (a float32 of magnitude below 2^62) to the nearest integer, halves away
-// from zero, with integer operations on its bits: y = m 2^e with m the 24-bit
-// significand, so the result is m << e, or (m + 2^(-e-1)) >> -e when e < 0.  (A
-// float-to-64-bit-integer conversion instruction runs on the FP64 pipe, which is
-// narrow on this GPU.)  Zero and subnormal inputs give 0.
-__device__ __forceinline__ long long fixed_round(float y) {
-  const unsigned b = __float_as_uint(y);
-  const int e = (int)((b >> 23) & 0xffu) - 150;
-  if (e < -24) return 0;                              // |y| < 0.5
-  const long long m = (long long)((b & 0x7fffffu) | 0x800000u);
-  const long long q = e >= 0 ? (m << e) : ((m + (1ll << (-e - 1))) >> (-e));
-  return (b >> 31) ? -q : q;
 }
 
 // One group of G lanes (G in {8, 16, 32}) processes one row bundle (layout.h):
@@ -269,18 +199,6 @@ __device__ __forceinline__ void process_bundle(const int4* __restrict__ rec, int
       }
     }
   }
-}
-
-// Scale exponent F of the fixed-point accumulation: 2^F * bound <= 2^60, so
-// that no sum of up to 2^2 times the bound (float32 rounding of the products
-// included) can overflow 63 bits; kFexpNaN marks a non-finite vector.
-__device__ __forceinline__ int fixed_exp(float vmax, double k, double pterm) {
-  if (!isfinite(vmax)) return kFexpNaN;
-  const double bound = k * (double)vmax + pterm;
-  if (!(bound > 0.0)) return 0;
-  int e;
-  frexp(bound, &e);                              // bound < 2^e
-  return max(-126, min(126, 60 - e));
 }
 
 // ---------------------------------------------------------------------------
@@ -826,6 +744,7 @@ size_t tma_smem_bytes(int n_pad, int cmax, int rmax, int stages, int value_bytes
 }
 
 void* rowpass_kernel(const DevPlan& P, int mode) {
+  if (use_priv(P)) return priv_rowpass_kernel(P, mode);
   switch (mode) {
     case kNormal: return pick<kNormal>(P);
     case kResid: return pick<kResid>(P);
@@ -839,6 +758,7 @@ size_t rowpass_smem(const DevPlan& P, int mode) {
   if (P.path == 1 || P.path == 3) {
     const int vb = P.value_format == 0 ? 4 : (P.value_format == 1 ? 2 : 1);
     const int ib = P.index_width == 16 ? 2 : 4;
+    if (use_priv(P)) return priv_fixed_bytes(P.n_pad, P.priv_acc, P.acc64 != 0) + (size_t)P.ring_bytes;
     return tma_smem_bytes(P.n_pad, P.cmax, P.rmax, P.stages, vb, ib, scatter, P.path == 3, P.acc64 != 0);
   }
   if (P.path == 2) return stream_smem_bytes(P.n_pad, P.rmax, scatter);
@@ -846,6 +766,7 @@ size_t rowpass_smem(const DevPlan& P, int mode) {
 }
 
 int rowpass_threads(const DevPlan& P) {
+  if (use_priv(P)) return priv_threads(P.priv);
   if (P.path == 3) return (P.ring_threads == 768 || P.ring_threads == 640) ? P.ring_threads : kTmaThreads;
   return P.path == 1 ? kTmaThreads : (P.path == 2 ? kStrThreads : kRowThreads);
 }

@@ -976,12 +976,13 @@ void launch(Exec& e, void (*fn)(A...), dim3 grid, dim3 block, size_t smem, A... 
   e.kernel((void*)fn, grid, block, smem, ptrs);
 }
 
+// objective: kResid passes also leave the per-scenario objective (kObj, kDose always do)
 void rowpass(Exec& e, Plan* P, int mode, const float* v, int v_stride, const int* active,
-             float* dose = nullptr) {
+             float* dose = nullptr, bool objective = true) {
   const DevPlan& dp = P->dp;
   void* fn = rowpass_kernel(dp, mode);
   float* partial = P->partial;
-  double* objp = P->objp;
+  double* objp = objective || !use_priv(dp) ? P->objp : nullptr;
   void* args[] = {(void*)&dp, (void*)&v, (void*)&v_stride, (void*)&active,
                   (void*)&partial, (void*)&objp, (void*)&dose};
   e.kernel(fn, dim3(dp.grid), dim3(rowpass_threads(dp)), rowpass_smem(dp, mode), args);
@@ -993,7 +994,7 @@ void admm_iteration_head(Exec& e, Plan* P, unsigned long long hcg, int uc) {
   const DevPlan& dp = P->dp;
   dim3 g2(P->nchunk, dp.N);
   // a batched plan skips the scenarios of problems that have stopped
-  rowpass(e, P, kResid, P->v32, dp.n_pad, dp.G > 1 ? P->uact : nullptr);
+  rowpass(e, P, kResid, P->v32, dp.n_pad, dp.G > 1 ? P->uact : nullptr, nullptr, /*objective=*/false);
   launch(e, k_cg_init, g2, dim3(VT), 0, dp, P->ctl, (const float*)P->partial, (const double*)P->x,
          (const double*)P->y, (const double*)P->z, (const double*)P->dinv, P->r, P->u, P->v32, P->dots,
          P->nchunk, P->gam, P->tol, P->r0n, P->act, P->cgi, P->cnt_s, hcg, uc);
