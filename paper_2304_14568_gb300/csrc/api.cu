@@ -858,7 +858,6 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
   P->beta = A.get<double>(N);
   P->bb_step = A.get<double>(N);
   P->act = A.get<int>(N);
-  P->act_next = A.get<int>(N);
   P->cgcnt = A.get<int>(N);
   P->cnt_s = A.get<unsigned int>(N);
   P->dots = A.get<double>((size_t)N * P->nchunk * 4);

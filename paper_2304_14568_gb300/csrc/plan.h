@@ -45,8 +45,8 @@ struct Ctl {
   int pgd_max_iter, max_trials, trial, accepted, failed, pk, pouter, pad2;
   long long trials_total;
   // last-block-done counters (every finisher resets its own counter)
-  unsigned int cnt_init, cnt_upd, cnt_d, cnt_y, cnt_z, cnt_red, cnt_pg, cnt_pt;
-  unsigned int pad3;
+  unsigned int cnt_init, cnt_d, cnt_y, cnt_z, cnt_red, cnt_pg, cnt_pt, pad3;
+  unsigned long long cnt_cg;       // CG step: scenarios done (low half) and going on (high half)
   // optional per-iteration trace (rpt_admm_params.trace): kTraceFields doubles per
   // iteration, at most trace_cap iterations, written by the dual update's last block
   double* trace;
@@ -99,7 +99,7 @@ struct Plan {
   double *gam = nullptr, *tol = nullptr, *r0n = nullptr, *alpha = nullptr, *beta = nullptr;
   double *bb_step = nullptr;      // [N] per-scenario ADMM dual steps
   double *gprev = nullptr, *aprev = nullptr;
-  int *act = nullptr, *act_next = nullptr, *cgcnt = nullptr, *cgi = nullptr;
+  int *act = nullptr, *cgcnt = nullptr, *cgi = nullptr;
   int *err = nullptr;             // device error word of the row passes
   unsigned int *cnt_s = nullptr;  // [N] per-scenario counters
   double *dots = nullptr;         // [N][nchunk][4]

@@ -16,6 +16,7 @@
 // Vectors are float64; the row passes see them rounded to float32 (staged in
 // shared memory).  Dot products and norms are float64; the per-CTA partials of
 // a row pass are summed in a fixed order with compensated float32 sums.
+#include <algorithm>
 #include <chrono>
 #include <cstddef>
 #include <cmath>
@@ -37,41 +38,53 @@ __device__ __forceinline__ double clampd(double v, double lo, double hi) {
   return fmin(fmax(v, lo), hi);
 }
 
-// Compensated sum, in the slot list's fixed order, of scenario s's row-pass
-// partials at column j; list holds the cnt slots of scenario s (in global or
-// shared memory, written before this kernel started).  Sixteen slots at a
-// time: all loads of a batch are issued before the (order-preserving) sums
+// Slots of scenario s's partial sums: consecutive from `first` for the pass with
+// private accumulators (list null), else listed.
+struct Slots {
+  const int* list;
+  int first, cnt;
+  __device__ __forceinline__ size_t at(int k) const { return (size_t)(list ? list[k] : first + k); }
+};
+__device__ __forceinline__ Slots slots_of(const DevPlan& P, int s) {
+  const int* list = P.slot_list + (size_t)s * P.slot_cap;
+  Slots S;
+  S.cnt = __ldcg(&P.slot_count[s]);
+  S.first = __ldcg(list);          // (unused but readable when cnt is 0)
+  S.list = P.priv ? nullptr : list;
+  return S;
+}
+
+// Compensated sum, in slot order, of scenario s's row-pass partials at column j.
+// Sixteen slots at a time, the last batch filled up with zeros (which change
+// nothing): all loads of a batch are issued before the (order-preserving) sums
 // consume them.
 __device__ __forceinline__ double sum_partials_of(const DevPlan& P, const float* __restrict__ part, int s, int j,
-                                                  const int* list, int cnt) {
+                                                  const Slots& S) {
   constexpr int kB = 16;
   if (P.acc64) {
     // bundled path: 64-bit fixed-point partials, summed exactly (every partial
     // and every sum stays below 2^62 in magnitude), then scaled by 2^-fexp[s]
     // and by the column scale of quantised values
     const long long* pl = reinterpret_cast<const long long*>(part);
+    const int fe = __ldcg(&P.fexp[s]);
     long long sum = 0;
-    int k = 0;
-    for (; k + kB <= cnt; k += kB) {
+    for (int k = 0; k < S.cnt; k += kB) {
       long long v[kB];
 #pragma unroll
-      for (int u = 0; u < kB; ++u) v[u] = __ldcg(pl + (size_t)list[k + u] * P.n_pad + j);
+      for (int u = 0; u < kB; ++u) v[u] = k + u < S.cnt ? __ldcg(pl + S.at(k + u) * P.n_pad + j) : 0ll;
 #pragma unroll
       for (int u = 0; u < kB; ++u) sum += v[u];
     }
-    for (; k < cnt; ++k) sum += __ldcg(pl + (size_t)list[k] * P.n_pad + j);
-    const int fe = __ldcg(&P.fexp[s]);
     if (fe == kFexpNaN) return __longlong_as_double(0x7ff8000000000000ll);
     double r = ldexp((double)sum, -fe);
     if (P.colscale) r *= (double)P.colscale[(size_t)s * P.n_pad + j];
     return r;
   }
   float sum = 0.f, c = 0.f;
-  int k = 0;
-  for (; k + kB <= cnt; k += kB) {
+  for (int k = 0; k < S.cnt; k += kB) {
     float v[kB];
 #pragma unroll
-    for (int u = 0; u < kB; ++u) v[u] = __ldcg(part + (size_t)list[k + u] * P.n_pad + j);
+    for (int u = 0; u < kB; ++u) v[u] = k + u < S.cnt ? __ldcg(part + S.at(k + u) * P.n_pad + j) : 0.f;
 #pragma unroll
     for (int u = 0; u < kB; ++u) {
       float t, e;
@@ -80,18 +93,11 @@ __device__ __forceinline__ double sum_partials_of(const DevPlan& P, const float*
       c += e;
     }
   }
-  for (; k < cnt; ++k) {
-    const float v = __ldcg(part + (size_t)list[k] * P.n_pad + j);
-    float t, e;
-    two_sum(sum, v, t, e);
-    sum = t;
-    c += e;
-  }
   return (double)sum + (double)c;
 }
 
 __device__ __forceinline__ double sum_partials(const DevPlan& P, const float* __restrict__ part, int s, int j) {
-  return sum_partials_of(P, part, s, j, P.slot_list + (size_t)s * P.slot_cap, __ldcg(&P.slot_count[s]));
+  return sum_partials_of(P, part, s, j, slots_of(P, s));
 }
 
 // Objective of the last objective pass: sum over scenarios (fixed order).
@@ -265,55 +271,64 @@ __global__ void k_cg_init(DevPlan P, Ctl* C, const float* __restrict__ partial,
   }
 }
 
-// grid (kCgCluster, N) in clusters of kCgCluster CTAs along x; the cluster of
-// scenario s makes one whole CG step after the operator pass:
+// grid (cluster, N), one cluster along x per scenario; it makes one whole CG step
+// after the operator pass:
 //   w = B u = (row-pass partials) + (rho/2) u;  delta = (w, u);  beta and alpha;
 //   p = u + beta p;  q = w + beta q;  x += alpha p;  r -= alpha q;  u = M^{-1} r (staged);
 //   gamma = (r, u), ||r||; activity; loop condition.
-// A CTA has kCgSub rows of kVecThreads threads; column chunk c (kVecThreads
-// columns) belongs to the cluster's CTA c mod kCgCluster, to its thread row
-// (c / kCgCluster) mod kCgSub and to its round c / (kCgCluster kCgSub), column
-// j to thread j mod kVecThreads of that row, and a thread takes its rounds in
-// increasing order; each CTA's sums are block reductions and the cluster's the
-// CTAs' sums added in rank order through distributed shared memory.  The order
-// depends on the column index only, not on n: the wider spot range of a
-// batched plan adds exact zeros.  w and u stay in registers between the two
-// halves; the cluster barriers are hardware barriers.
+// Column chunk c (kVecThreads columns) belongs to the cluster's CTA c mod
+// kCgCluster, to its thread row (c / kCgCluster) mod kCgSub and to its round c /
+// (kCgCluster kCgSub), column j to thread j mod kVecThreads of that row, and a
+// thread takes its rounds in increasing order; each CTA's sums are block
+// reductions and the cluster's the CTAs' sums added in rank order.  CTAs and thread
+// rows that no column falls to are not launched (cg_shape): they would add exact
+// zeros, so the result depends on the column index only, not on n, and a problem
+// in a batched plan of more spots follows its own plan bit for bit.  w and u stay
+// in registers between the two halves; the cluster barriers are hardware barriers.
+// Bound: the chain of latencies (scalars, slots, partials, two cluster barriers,
+// one counter).  The scenario's scalars and slots are loaded together; every CTA
+// sends its part of a sum to the shared memory that reads it, so a barrier is
+// followed by local loads only; the counter that finds the last scenario to finish
+// also adds up how many go on.  A CG step with its pass, the rest of an iteration
+// included: 250 spots, 13 scenarios 36 us before and 28 us after; 52 units of 250
+// to 550 spots 150 us before and 112 us after.
 constexpr int kCgCluster = 8;
 constexpr int kCgSub = 4;
 constexpr int kCgThreads = kCgSub * kVecThreads;
 constexpr int kCgChunks = (RPT_MAX_SPOTS + kCgThreads * kCgCluster - 1) / (kCgThreads * kCgCluster);
 constexpr int kErrCgCluster = 16;   // error word: the CG step ran without its cluster
-constexpr int kCgListCap = 2048;    // slot lists up to this length are read from shared memory
 
-__global__ void __cluster_dims__(kCgCluster, 1, 1) __launch_bounds__(kCgThreads, 1)
+// CTAs per cluster (a power of two) and threads per CTA for n columns.
+inline void cg_shape(int n, int* cluster, int* threads) {
+  const int chunks = (n + kVecThreads - 1) / kVecThreads;
+  *cluster = 1;
+  while (*cluster < chunks && *cluster < kCgCluster) *cluster *= 2;
+  *threads = kVecThreads * std::min(kCgSub, (chunks + kCgCluster - 1) / kCgCluster);
+}
+
+__global__ void __launch_bounds__(kCgThreads, 1)
 k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double* q,
           const float* __restrict__ partial, const double* __restrict__ dinv, float* v32, double* gam,
-          double* gprev, double* aprev, const double* __restrict__ tol, int* act, int* act_next, int* cgi,
+          double* gprev, double* aprev, const double* __restrict__ tol, int* act, int* cgi,
           int* cgcnt, unsigned long long hcg, int use_cond) {
   __shared__ double sh[2 * 32];
-  __shared__ double cl_part[3];   // this CTA's parts of delta, gamma and ||r||^2 (read by the cluster)
+  __shared__ double part1[kCgCluster], part2[2 * kCgCluster];   // the cluster's parts of delta; of gamma and ||r||^2
   __shared__ double ab[2];
-  __shared__ int s_list[kCgListCap];
   cg::cluster_group cl = cg::this_cluster();
-  if (cl.num_blocks() != kCgCluster) {   // never expected: report it and touch nothing
+  const int nr = (int)gridDim.x;
+  if ((int)cl.num_blocks() != nr) {   // never expected: report it and touch nothing
     if (threadIdx.x == 0) atomicExch(P.err, kErrCgCluster);
     return;
   }
   const int s = blockIdx.y, rank = (int)cl.block_rank();
   const int sub = threadIdx.x / VT, col = threadIdx.x % VT;
-  if (__ldcg(&act[s]) == 0) return;      // the same answer in every CTA of the cluster
+  // all loads in flight together; rank 0 rewrites act, cgi and the scalars only
+  // after every CTA of the cluster has passed both barriers
+  const int active = __ldcg(&act[s]);
   const int any = __ldcg(&C->cg_any);
   const bool first = __ldcg(&cgi[s]) == 0;
   const double hr = 0.5 * C->g[s / P.Ns].rho;
-  // the scenario's slot list into shared memory, and the step's scalars, all
-  // loads in flight together (this kernel's rank 0 rewrites the scalars only
-  // after every CTA of the cluster has passed its second barrier)
-  const int cnt = __ldcg(&P.slot_count[s]);
-  const int* glist = P.slot_list + (size_t)s * P.slot_cap;
-  const int* list = cnt <= kCgListCap ? s_list : glist;
-  if (cnt <= kCgListCap)
-    for (int k = threadIdx.x; k < cnt; k += blockDim.x) s_list[k] = __ldcg(&glist[k]);
+  const Slots slots = slots_of(P, s);
   double g_s = 0.0, gp_s = 0.0, ap_s = 0.0, tol_s = 0.0;
   if (threadIdx.x == 0) {
     g_s = __ldcg(&gam[s]);
@@ -321,19 +336,22 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
     ap_s = __ldcg(&aprev[s]);
     tol_s = __ldcg(&tol[s]);
   }
-  __syncthreads();
-  double uv[kCgChunks], wv[kCgChunks];
-  // the second half's operands of the first round are loaded now, so that
-  // their latency overlaps the first half's sums and barriers
+  // the operands of the first round are loaded now, so that their latency
+  // overlaps the first half's sums and barriers
   const int j0 = (sub * kCgCluster + rank) * VT + col;
   const size_t o0 = (size_t)s * P.n + j0;
-  double p0 = 0.0, q0 = 0.0, r0 = 0.0, d0 = 0.0;
+  double u0 = 0.0, p0 = 0.0, q0 = 0.0, r0 = 0.0, d0 = 0.0, x0 = 0.0;
   if (j0 < P.n) {
+    u0 = u[o0];
     p0 = p[o0];
     q0 = q[o0];
     r0 = r[o0];
     d0 = dinv[o0];
+    x0 = x[o0];
   }
+  // the same answer in every CTA of the cluster (the loop is over: a further step of the loop body)
+  if (active == 0 || any == 0 || __ldcg(&C->kcg) >= C->cg_max) return;
+  double uv[kCgChunks], wv[kCgChunks];
   double dl[1] = {0.0};
 #pragma unroll
   for (int t = 0; t < kCgChunks; ++t) {
@@ -341,22 +359,17 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
     uv[t] = 0.0;
     wv[t] = 0.0;
     if (j < P.n) {
-      const size_t o = (size_t)s * P.n + j;
-      uv[t] = u[o];
-      wv[t] = sum_partials_of(P, partial, s, j, list, cnt) + hr * uv[t];
+      uv[t] = t == 0 ? u0 : u[(size_t)s * P.n + j];
+      wv[t] = sum_partials_of(P, partial, s, j, slots) + hr * uv[t];
       dl[0] += wv[t] * uv[t];
     }
   }
   block_sum_d<1>(dl, sh);
-  if (threadIdx.x == 0) cl_part[0] = dl[0];
+  if ((int)threadIdx.x < nr) *cl.map_shared_rank(&part1[rank], (int)threadIdx.x) = dl[0];   // (valid in warp 0)
   cl.sync();
   if (threadIdx.x == 0) {
-    double parts[kCgCluster];
-#pragma unroll
-    for (int k = 0; k < kCgCluster; ++k) parts[k] = *cl.map_shared_rank(&cl_part[0], k);
     double delta = 0.0;
-#pragma unroll
-    for (int k = 0; k < kCgCluster; ++k) delta += parts[k];
+    for (int k = 0; k < nr; ++k) delta += part1[k];
     const double b = first ? 0.0 : g_s / gp_s;
     const double den = first ? delta : delta - b * g_s / ap_s;
     ab[0] = (den > 0.0 && isfinite(den) && isfinite(b)) ? g_s / den : 0.0;
@@ -374,7 +387,7 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
       const double qj = first ? wv[t] : fma(b, t == 0 ? q0 : q[o], wv[t]);
       p[o] = pj;
       q[o] = qj;
-      x[o] = fma(a, pj, x[o]);
+      x[o] = fma(a, pj, t == 0 ? x0 : x[o]);
       const double rj = fma(-a, qj, t == 0 ? r0 : r[o]);
       const double uj = (t == 0 ? d0 : dinv[o]) * rj;
       r[o] = rj;
@@ -385,57 +398,34 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
     }
   }
   block_sum_d<2>(v, sh);
-  if (threadIdx.x == 0) {
-    cl_part[1] = v[0];
-    cl_part[2] = v[1];
-  }
+  if (threadIdx.x < 2) *cl.map_shared_rank(&part2[2 * rank + threadIdx.x], 0) = threadIdx.x ? v[1] : v[0];
   cl.sync();
-  if (rank == 0 && threadIdx.x == 0) {
-    double pg[kCgCluster], pr[kCgCluster];
-#pragma unroll
-    for (int k = 0; k < kCgCluster; ++k) {
-      pg[k] = *cl.map_shared_rank(&cl_part[1], k);
-      pr[k] = *cl.map_shared_rank(&cl_part[2], k);
-    }
-    double g = 0.0, rr = 0.0;
-#pragma unroll
-    for (int k = 0; k < kCgCluster; ++k) {
-      g += pg[k];
-      rr += pr[k];
-    }
-    gprev[s] = g_s;
-    aprev[s] = a;
-    gam[s] = g;
-    cgi[s] += 1;
-    cgcnt[s] += 1;
-    act_next[s] = (a > 0.0 && g > 0.0 && sqrt(rr) > tol_s) ? 1 : 0;
+  if (rank != 0 || threadIdx.x != 0) return;
+  double g = 0.0, rr = 0.0;
+  for (int k = 0; k < nr; ++k) {
+    g += part2[2 * k];
+    rr += part2[2 * k + 1];
   }
-  cl.sync();   // every CTA's shared memory stays until rank 0 has read it
-  if (rank != 0) return;
-  // rank 0 of every stepping scenario; the last to arrive ends the step
-  if (!last_block(&C->cnt_upd, (unsigned int)any) || threadIdx.x >= 32) return;
-  // warp 0: the scenarios of this step (lane l takes l, l + 32, ...) count one CG
-  // step each and take their next activity
-  int was = 0, na = 0;
-  for (int k = threadIdx.x; k < P.N; k += 32) {
-    const int ak = __ldcg(&act[k]), nx = __ldcg(&act_next[k]);   // both loads in flight
-    if (ak) {
-      ++was;
-      atomicAdd(reinterpret_cast<unsigned long long*>(&C->g[k / P.Ns].cg), 1ull);
-      act[k] = nx;
-      na += nx;
-    }
-  }
-  was = __reduce_add_sync(0xffffffffu, was);
-  na = __reduce_add_sync(0xffffffffu, na);
-  if (threadIdx.x == 0) {
-    C->cg_total += was;
-    C->cg_any = na;
-    C->kcg += 1;
-    C->cg_steps += 1;
-    C->passes += 1;
-    set_cond(hcg, use_cond, na > 0 && C->kcg < C->cg_max);
-  }
+  const int next = (a > 0.0 && g > 0.0 && sqrt(rr) > tol_s) ? 1 : 0;
+  gprev[s] = g_s;
+  aprev[s] = a;
+  gam[s] = g;
+  cgi[s] += 1;
+  cgcnt[s] += 1;
+  act[s] = next;
+  atomicAdd(reinterpret_cast<unsigned long long*>(&C->g[s / P.Ns].cg), 1ull);
+  // the last of the step's `any` scenarios ends it: low half the scenarios done,
+  // high half those that go on
+  const unsigned long long done = atomicAdd(&C->cnt_cg, 1ull | ((unsigned long long)next << 32));
+  if ((int)(done & 0xffffffffull) + 1 != any) return;
+  const int na = (int)(done >> 32) + next;
+  C->cnt_cg = 0ull;
+  C->cg_total += any;
+  C->cg_any = na;
+  C->kcg += 1;
+  C->cg_steps += 1;
+  C->passes += 1;
+  set_cond(hcg, use_cond, na > 0 && C->kcg < C->cg_max);
 }
 
 // grid (nchunk, G).  Per group: z_new = P_box(mean_s(x_s + y_s/rho)) [std] or
@@ -724,16 +714,38 @@ __global__ void k_pgd_init(DevPlan P, const double* __restrict__ x0, int has_x0,
   }
 }
 
-// grid (nchunk).  g = 2 sum_s A~_s^T (A~_s x - p~) (Eq. 4 summed over s) from a kResid
-// pass over all scenarios; f(x); start the Armijo trials at t = alpha.
-__global__ void k_pgd_grad(DevPlan P, Ctl* C, const float* __restrict__ partial,
-                           double* g, unsigned long long htrial, int use_cond) {
-  const int j = blockIdx.x * VT + threadIdx.x;
-  if (j < P.n) {
-    double gj = 0.0;
-    for (int s = 0; s < P.N; ++s) gj += sum_partials(P, partial, s, j);
-    g[j] = 2.0 * gj;
+// Sum over all scenarios of the row-pass partials, for 32 columns per block of 32 x
+// kAllRows threads: latency-bound, so thread row y takes scenarios y, y + kAllRows,
+// ... (kAllRows at a time, into shared memory) and row 0 adds each batch in
+// scenario order.  True in the threads that hold a column's sum.  1777 spots, 7
+// scenarios: 5 us against 38 us for one thread per column.
+constexpr int kAllRows = 16;
+__device__ __forceinline__ bool sum_all_scenarios(const DevPlan& P, const float* __restrict__ part, int& j,
+                                                  double& sum) {
+  __shared__ double sh[kAllRows][33];
+  const int c = threadIdx.x & 31, y = threadIdx.x >> 5;
+  j = blockIdx.x * 32 + c;
+  sum = 0.0;
+  for (int s0 = 0; s0 < P.N; s0 += kAllRows) {
+    const int s = s0 + y;
+    const double v = (s < P.N && j < P.n) ? sum_partials(P, part, s, j) : 0.0;
+    __syncthreads();
+    sh[y][c] = v;
+    __syncthreads();
+    if (y == 0)
+      for (int k = 0; k < kAllRows && s0 + k < P.N; ++k) sum += sh[k][c];
   }
+  return y == 0 && j < P.n;
+}
+
+// grid (ceil(n / 32)).  g = 2 sum_s A~_s^T (A~_s x - p~) (Eq. 4 summed over s) from a kResid
+// pass over all scenarios; f(x); start the Armijo trials at t = alpha.
+__global__ void __launch_bounds__(32 * kAllRows)
+k_pgd_grad(DevPlan P, Ctl* C, const float* __restrict__ partial,
+           double* g, unsigned long long htrial, int use_cond) {
+  int j;
+  double gj;
+  if (sum_all_scenarios(P, partial, j, gj)) g[j] = 2.0 * gj;
   if (!last_block(&C->cnt_pg, gridDim.x)) return;
   if (threadIdx.x == 0) {
     C->fx = objective_sum(P) + C->const_term;
@@ -907,13 +919,12 @@ k_chol_x(DevPlan P, const Ctl* __restrict__ C, const float* __restrict__ binv, c
   }
 }
 
-// grid (nchunk): out = scale * sum over all blocks.
-__global__ void k_reduce_all(DevPlan P, const float* __restrict__ partial, double scale, double* out) {
-  const int j = blockIdx.x * VT + threadIdx.x;
-  if (j >= P.n) return;
-  double v = 0.0;
-  for (int s = 0; s < P.N; ++s) v += sum_partials(P, partial, s, j);
-  out[j] = scale * v;
+// grid (ceil(n / 32)): out = scale * sum over all scenarios.
+__global__ void __launch_bounds__(32 * kAllRows)
+k_reduce_all(DevPlan P, const float* __restrict__ partial, double scale, double* out) {
+  int j;
+  double v;
+  if (sum_all_scenarios(P, partial, j, v)) out[j] = scale * v;
 }
 
 // ---------------------------------------------------------------------------
@@ -929,10 +940,26 @@ struct Exec {
 
   bool graph() const { return g != nullptr; }
 
-  void kernel(void* fn, dim3 grid, dim3 block, size_t smem, void** args) {
+  // cluster: CTAs per thread-block cluster along x (1: none asked for)
+  void kernel(void* fn, dim3 grid, dim3 block, size_t smem, void** args, int cluster = 1) {
     if (err != cudaSuccess) return;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
     if (!graph()) {
-      err = cudaLaunchKernel(fn, grid, block, args, smem, st);
+      if (cluster == 1) {
+        err = cudaLaunchKernel(fn, grid, block, args, smem, st);
+        return;
+      }
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = grid;
+      cfg.blockDim = block;
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = st;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      err = cudaLaunchKernelExC(&cfg, fn, args);
       return;
     }
     cudaKernelNodeParams kp{};
@@ -943,6 +970,7 @@ struct Exec {
     kp.kernelParams = args;
     cudaGraphNode_t node;
     err = cudaGraphAddKernelNode(&node, g, last ? &last : nullptr, last ? 1 : 0, &kp);
+    if (err == cudaSuccess && cluster > 1) err = cudaGraphKernelNodeSetAttribute(node, at.id, &at.val);
     if (err == cudaSuccess) last = node;
   }
 
@@ -976,6 +1004,12 @@ void launch(Exec& e, void (*fn)(A...), dim3 grid, dim3 block, size_t smem, A... 
   e.kernel((void*)fn, grid, block, smem, ptrs);
 }
 
+template <typename... A>
+void launch_cluster(Exec& e, int cluster, void (*fn)(A...), dim3 grid, dim3 block, size_t smem, A... args) {
+  void* ptrs[] = {(void*)&args...};
+  e.kernel((void*)fn, grid, block, smem, ptrs, cluster);
+}
+
 // objective: kResid passes also leave the per-scenario objective (kObj, kDose always do)
 void rowpass(Exec& e, Plan* P, int mode, const float* v, int v_stride, const int* active,
              float* dose = nullptr, bool objective = true) {
@@ -1003,9 +1037,11 @@ void admm_iteration_head(Exec& e, Plan* P, unsigned long long hcg, int uc) {
 void cg_body(Exec& e, Plan* P, unsigned long long hcg, int uc) {
   const DevPlan& dp = P->dp;
   rowpass(e, P, kNormal, P->v32, dp.n_pad, P->act);
-  launch(e, k_cg_step, dim3(kCgCluster, dp.N), dim3(kCgThreads), 0, dp, P->ctl, P->x, P->r, P->u, P->p, P->q,
-         (const float*)P->partial, (const double*)P->dinv, P->v32, P->gam, P->gprev, P->aprev,
-         (const double*)P->tol, P->act, P->act_next, P->cgi, P->cgcnt, hcg, uc);
+  int cluster, threads;
+  cg_shape(dp.n, &cluster, &threads);
+  launch_cluster(e, cluster, k_cg_step, dim3(cluster, dp.N), dim3(threads), 0, dp, P->ctl, P->x, P->r, P->u, P->p,
+                 P->q, (const float*)P->partial, (const double*)P->dinv, P->v32, P->gam, P->gprev, P->aprev,
+                 (const double*)P->tol, P->act, P->cgi, P->cgcnt, hcg, uc);
 }
 
 void admm_iteration_tail(Exec& e, Plan* P, int use_obj, unsigned long long hadmm, int uc, ConHook* con = nullptr) {
@@ -1068,6 +1104,12 @@ cudaError_t build_admm_chol_graph(Plan* P, int use_obj) {
   return err;
 }
 
+// CG steps per pass of the CG loop's body: the loop node costs about 2 us a pass,
+// and a step after the last one finds no active scenario (its row pass has no
+// work).  250 spots, 30 iterations: 8.44 ms with one, 8.16 with two; realistic plan,
+// 12 iterations: 33.9 and 33.6 ms; three and four gain no more.
+constexpr int kCgUnroll = 2;
+
 cudaError_t build_admm_graph(Plan* P, int use_obj, double* z0d, double* y0d) {
   (void)z0d;
   (void)y0d;
@@ -1084,7 +1126,7 @@ cudaError_t build_admm_graph(Plan* P, int use_obj, double* z0d, double* y0d) {
     body.err = cudaGraphConditionalHandleCreate(&hcg, body.g, 0, cudaGraphCondAssignDefault);
   admm_iteration_head(body, P, (unsigned long long)hcg, 1);
   Exec cg = body.while_body(hcg);
-  cg_body(cg, P, (unsigned long long)hcg, 1);
+  for (int k = 0; k < kCgUnroll; ++k) cg_body(cg, P, (unsigned long long)hcg, 1);
   if (cg.err != cudaSuccess) body.err = cg.err;
   admm_iteration_tail(body, P, use_obj, (unsigned long long)hadmm, 1);
   if (body.err != cudaSuccess) top.err = body.err;
@@ -1105,7 +1147,7 @@ cudaError_t build_admm_graph(Plan* P, int use_obj, double* z0d, double* y0d) {
 void pgd_head(Exec& e, Plan* P, unsigned long long htrial, int uc) {
   const DevPlan& dp = P->dp;
   rowpass(e, P, kResid, P->vz32, 0, nullptr);
-  launch(e, k_pgd_grad, dim3(P->nchunk), dim3(VT), 0, dp, P->ctl, (const float*)P->partial,
+  launch(e, k_pgd_grad, dim3((dp.n + 31) / 32), dim3(32 * kAllRows), 0, dp, P->ctl, (const float*)P->partial,
          P->g, htrial, uc);
 }
 
@@ -1414,7 +1456,8 @@ int admm_solve_impl(Plan* P, const rpt_admm_params* prm, const double* z0, const
     if ((e = cudaStreamSynchronize(st))) return cuda_fail(e, "sync");
   }
   // init + per iteration (residual pass, CG init, 2 per CG step, z/d/y, 2 for the
-  // optional objective test) + final objective pass and its reduction (+ staging)
+  // optional objective test) + final objective pass and its reduction (+ staging);
+  // the empty step that may end a CG loop in the graph is not counted
   const long long kernels = (chol ? 3 + 5LL * h.k : 3 + 5LL * h.k + 2LL * h.cg_steps) +
                             (use_obj ? 2LL * h.k : 0LL) + (G > 1 ? 1 : 0);
   auto fill = [&](rpt_solve_info* o, const Grp& q, int st_q) {
@@ -1617,7 +1660,7 @@ int op_gradient(Plan* P, const double* x, double* g_out, double* f_out) {
   Exec ex;
   ex.st = P->stream;
   rowpass(ex, P, kResid, P->vz32, 0, nullptr);
-  launch(ex, k_reduce_all, dim3(P->nchunk), dim3(VT), 0, dp, (const float*)P->partial, 2.0, P->g);
+  launch(ex, k_reduce_all, dim3((dp.n + 31) / 32), dim3(32 * kAllRows), 0, dp, (const float*)P->partial, 2.0, P->g);
   if (ex.err) return cuda_fail(ex.err, "launch");
   std::vector<double> objp(dp.N);
   if ((e = cudaMemcpyAsync(g_out, P->g, sizeof(double) * dp.n, cudaMemcpyDeviceToHost, P->stream)))
@@ -1746,7 +1789,7 @@ int compute_lipschitz(Plan* P, double* L) {
     Exec ex;
     ex.st = P->stream;
     rowpass(ex, P, kNormal, P->vz32, 0, nullptr);
-    launch(ex, k_reduce_all, dim3(P->nchunk), dim3(VT), 0, dp, (const float*)P->partial, 1.0, P->g);
+    launch(ex, k_reduce_all, dim3((dp.n + 31) / 32), dim3(32 * kAllRows), 0, dp, (const float*)P->partial, 1.0, P->g);
     if (ex.err) return cuda_fail(ex.err, "launch");
     if ((e = cudaMemcpyAsync(u.data(), P->g, sizeof(double) * dp.n, cudaMemcpyDeviceToHost, P->stream)))
       return cuda_fail(e, "copy");
