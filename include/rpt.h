@@ -148,7 +148,7 @@ typedef struct {
                              operator; RPT_SUB_CHOL the cached factor: B_s = A~_s^T A~_s + (rho/2) I
                              formed, factored and inverted once per (plan, rho) in FP32 on the device,
                              then x_s = B_s^{-1} c_s each iteration (4 n^2 N bytes of device memory,
-                             plus as much again while it is formed) */
+                             plus as much again for the workspace it is formed in) */
   int32_t trace;          /* 1: record one entry per iteration (see rpt_trace_get); default 0 */
   int32_t bb_per_scenario;/* 0 (default): one dual step over the concatenated vectors (Eq. 8 as
                              written); 1: Eq. 8 applied to each scenario's own blocks dd_s, dy_s,
@@ -247,7 +247,8 @@ int rpt_plan_create(const rpt_problem* prob, const rpt_device_opts* opts, rpt_pl
  * state (rpt_state_get) is kept.  The row passes then compute what a plan
  * created with these weights computes (the Jacobi diagonal and the default rho
  * may differ from a fresh plan's in the last bits, as they are summed in
- * another order).  Allocates and frees temporary device memory.  RPT_EINVAL
+ * another order).  The first call allocates a workspace on the device (8 bytes per
+ * spot and scenario and 16 per kept row), which the plan keeps.  RPT_EINVAL
  * for null or invalid arrays. */
 int rpt_plan_set_weights(rpt_plan* plan, const double* voxel_w, const double* presc);
 

@@ -1358,45 +1358,63 @@ int rpt_plan_set_weights(rpt_plan* plan, const double* voxel_w, const double* pr
       pk[k] = presc[P->kept_rows[k]];
       wmax = std::max(wmax, wk[k]);
     }
-    double* d = nullptr;                     // [wk | pk] then the fixed-point sums
-    cudaError_t e = cudaMalloc(&d, sizeof(double) * (2 * (size_t)m_act + n_pad));
-    if (e != cudaSuccess) return cuda_fail(e, "rpt_plan_set_weights");
-    unsigned long long* acc = reinterpret_cast<unsigned long long*>(d + 2 * (size_t)m_act);
-    e = cudaMemcpyAsync(d, wk.data(), sizeof(double) * m_act, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d + m_act, pk.data(), sizeof(double) * m_act, cudaMemcpyHostToDevice, st);
-    std::vector<unsigned long long> h(n_pad);
-    std::vector<float> diag((size_t)N * n);
-    double tr = 0.0;
-    for (int s = 0; s < N && e == cudaSuccess; ++s) {
+    // device: [wk | pk | c_s | scales] then the fixed-point sums of every scenario;
+    // kept by the plan, as weight sweeps call this again and again
+    const size_t in = 2 * (size_t)m_act + 2 * (size_t)N;
+    cudaError_t e = cudaSuccess;
+    if (!P->reweight) {
+      const size_t count = std::max(in + (size_t)N * n_pad, 2 * (size_t)n_pad);
+      if ((e = cudaMalloc(&P->reweight, sizeof(double) * count)) != cudaSuccess) {
+        P->reweight = nullptr;
+        return cuda_fail(e, "rpt_plan_set_weights");
+      }
+      P->allocs.push_back(P->reweight);
+    }
+    double* d = P->reweight;
+    unsigned long long* acc = reinterpret_cast<unsigned long long*>(d + in);
+    std::vector<double> sc(2 * (size_t)N);   // c_s, then the scales
+    for (int s = 0; s < N; ++s) {
       // sum_i c_s w_i a_ij^2 <= c_s max(w) max_j sum_i a_ij^2: scale so that 4x that stays below 2^62
       const double bound = P->scen_c[s] * wmax * P->colsq_max[s] * 4.0;
       int ex = 0;
       if (bound > 0.0) std::frexp(bound, &ex);
-      const double scale = std::ldexp(1.0, 60 - ex);
-      e = plan_reweight(P->dp, s, P->scen_c[s], d, d + m_act, scale, acc, st);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), acc, sizeof(unsigned long long) * n_pad,
-                                                cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      sc[s] = P->scen_c[s];
+      sc[N + s] = std::ldexp(1.0, 60 - ex);
+    }
+    e = cudaMemcpyAsync(d, wk.data(), sizeof(double) * m_act, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d + m_act, pk.data(), sizeof(double) * m_act, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(d + 2 * (size_t)m_act, sc.data(), sizeof(double) * sc.size(), cudaMemcpyHostToDevice, st);
+    const int blocks = std::max(1, (8 * P->sm_count + N - 1) / N);
+    if (e == cudaSuccess)
+      e = plan_reweight(P->dp, d + 2 * (size_t)m_act, d, d + m_act, d + 2 * (size_t)m_act + N, acc, blocks, st);
+    std::vector<unsigned long long> h((size_t)N * n_pad);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(h.data(), acc, sizeof(unsigned long long) * h.size(), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    std::vector<float> diag((size_t)N * n);
+    double tr = 0.0;
+    for (int s = 0; s < N; ++s)
       for (int j = 0; j < n; ++j) {   // each sum is exact; the trace adds them in column order
-        const double dj = (double)(long long)h[j] / scale;
+        const double dj = (double)(long long)h[(size_t)s * n_pad + j] / sc[N + s];
         diag[(size_t)s * n + j] = (float)dj;
         tr += dj;
       }
-    }
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(P->diag, diag.data(), sizeof(float) * diag.size(), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && P->dp.path == 3) e = bundle_bounds(P->dp, d, d + n_pad, const_cast<double*>(P->dp.kbound), st);
+    // the fixed-point bounds of exact-sum plans (the sums' space serves as scratch)
+    if (e == cudaSuccess && P->dp.acc64) e = bundle_bounds(P->dp, d, d + n_pad, const_cast<double*>(P->dp.kbound), st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(d);
     if (e != cudaSuccess) return cuda_fail(e, "rpt_plan_set_weights");
     // the constant of Eq. 2 in the order plan creation sums it
     double c = 0.0;
+    // (a voxel without a prescription adds nothing to it)
     for (int32_t i : P->dropped_rows)
-      for (int s = 0; s < N; ++s) c += P->scen_c[s] * voxel_w[i] * presc[i] * presc[i];
+      for (int s = 0; s < N && presc[i] != 0.0; ++s) c += P->scen_c[s] * voxel_w[i] * presc[i] * presc[i];
     for (int s = 0; s < N; ++s)
       for (int32_t k : P->empty_kept[s]) {
         const int32_t i = P->kept_rows[k];
-        c += P->scen_c[s] * voxel_w[i] * presc[i] * presc[i];
+        if (presc[i] != 0.0) c += P->scen_c[s] * voxel_w[i] * presc[i] * presc[i];
       }
     P->stats.const_term = c;
     P->stats.default_rho = 2.0 * (tr / N) / n;

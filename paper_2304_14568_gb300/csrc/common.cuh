@@ -178,9 +178,9 @@ size_t priv_fixed_bytes(int n_pad, int accs, bool fixed);   // shared memory bef
 // Bundled layout, at plan creation: kbound[2s], kbound[2s+1] of every scenario
 // (DevPlan::kbound) from the stored values; kc, pc: scratch [n_pad] doubles.
 cudaError_t bundle_bounds(const DevPlan& P, double* kc, double* pc, double* kbound, cudaStream_t st);
-// New weights for scenario s (rpt_plan_set_weights): rewrite its row records from
-// wk, pk (per kept row) and c_s, and add sum_i c_s w_i a_ij^2 * scale to acc
-// (int64 fixed point, [n_pad], zeroed here).
-cudaError_t plan_reweight(const DevPlan& P, int s, double cs, const double* wk, const double* pk, double scale,
-                          unsigned long long* acc, cudaStream_t st);
+// New weights (rpt_plan_set_weights): rewrite every scenario's row records from wk,
+// pk (per kept row) and cs [N], and sum_i c_s w_i a_ij^2 * scale[s] into acc (int64
+// fixed point, [N][n_pad], zeroed here); blocks: CTAs per scenario.  All on the device.
+cudaError_t plan_reweight(const DevPlan& P, const double* cs, const double* wk, const double* pk,
+                          const double* scale, unsigned long long* acc, int blocks, cudaStream_t st);
 }  // namespace rpt

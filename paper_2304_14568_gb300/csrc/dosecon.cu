@@ -107,7 +107,8 @@ __global__ void k_con_gtg(DevPlan P, ConDev D, float* __restrict__ B) {
   row_range(P, s, rw.x, BUN, lo, hi);
   const int len = hi - lo;
   const long long pairs = (long long)len * len;
-  float* Bs = B + (size_t)s * D.n * D.n;
+  const int ld = chol_ld(D.n);
+  float* Bs = B + (size_t)s * D.n * ld;
   for (long long p = threadIdx.x; p < pairs; p += blockDim.x) {
     const int e1 = lo + (int)(p / len), e2 = lo + (int)(p % len);
     int c1, c2;
@@ -115,7 +116,7 @@ __global__ void k_con_gtg(DevPlan P, ConDev D, float* __restrict__ B) {
     row_entry<VT, IT, BUN>(P, s, e1, rw.y, c1, a1);
     row_entry<VT, IT, BUN>(P, s, e2, rw.y, c2, a2);
     if (c1 < c2 || a1 == 0.0 || a2 == 0.0) continue;
-    atomicAdd(&Bs[(size_t)c1 * D.n + c2], (float)(0.5 * D.sigma * a1 * a2));
+    atomicAdd(&Bs[(size_t)c1 * ld + c2], (float)(0.5 * D.sigma * a1 * a2));
   }
 }
 
@@ -124,7 +125,8 @@ __global__ void k_con_gtg_mean(ConDev D, float* __restrict__ B) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
   if (j >= D.n || D.Km == 0) return;
   const double* G = D.gmean + (size_t)s * D.Km * D.n;
-  float* row = B + (size_t)s * D.n * D.n + (size_t)j * D.n;
+  const int ld = chol_ld(D.n);
+  float* row = B + (size_t)s * D.n * ld + (size_t)j * ld;
   for (int k = 0; k <= j; ++k) {
     double acc = 0.0;
     for (int c = 0; c < D.Km; ++c) acc += G[(size_t)c * D.n + j] * G[(size_t)c * D.n + k];

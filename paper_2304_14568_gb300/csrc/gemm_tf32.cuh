@@ -15,7 +15,11 @@
 // with the structure flags of gemm.cuh:
 //   lower: compute only output tiles that reach the lower triangle (j <= i);
 //   kdiag 1: op(B)(k, j) is zero for k < j (K starts at the tile's first column);
-//   kdiag 2: also op(A)(i, k) is zero for k < i (K starts at max of both).
+//   kdiag 2: also op(A)(i, k) is zero for k < i (K starts at max of both);
+//   kdiag 3: op(A)(i, k) is zero for k < i (K starts at the tile's first row);
+//   kdiag 4: op(A)(i, k) is zero for k > i (K ends with the tile's last row).
+// Several products per batch entry (T3Pairs): product p of an entry works p steps
+// further along, and the last one may be cut short.
 // A CTA computes a 64 x 64 tile with 4 warps of 32 x 32 (2 x 4 mma tiles each);
 // K advances in steps of 32 staged in shared memory as [row][k] for op(A) and
 // [column][k] for op(B) (a row stride of 36 floats keeps the fragment loads of a
@@ -23,6 +27,7 @@
 // memory into registers while the tensor cores work on the current one.
 // beta == 0 never reads C.
 #pragma once
+#include <algorithm>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -52,19 +57,38 @@ __device__ __forceinline__ void mma_tf32_m16n8k8(float (&d)[4], const uint32_t (
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
+// blockIdx.z = entry * count + p: A, B, C move by `step` elements per p; product p
+// has at most `rows - p * rows_step` of the extent that is ragged (1: M and K, 2: N)
+struct T3Pairs {
+  int count = 1;
+  long long step = 0;
+  int rows = 0, rows_step = 0, ragged = 0;
+};
+
 template <bool TA, bool TB>
 __global__ void __launch_bounds__(kT3Threads)
-k_gemm_tf32x3(int M, int N, int K, const float* __restrict__ A, int lda, long long sA, const float* __restrict__ B,
-              int ldb, long long sB, float* __restrict__ C, int ldc, long long sC, float alpha, float beta,
-              int lower, int kdiag) {
+k_gemm_tf32x3(int M, int N, int K, const float* A, int lda, long long sA, const float* B,
+              int ldb, long long sB, float* C, int ldc, long long sC, float alpha, float beta,
+              int lower, int kdiag, T3Pairs pr) {
   __shared__ __align__(16) float As[kT3BM][kT3BK + kT3Pad];
   __shared__ __align__(16) float Bs[kT3BN][kT3BK + kT3Pad];
-  A += (long long)blockIdx.z * sA;
-  B += (long long)blockIdx.z * sB;
-  C += (long long)blockIdx.z * sC;
+  const int ent = pr.count == 1 ? (int)blockIdx.z : (int)blockIdx.z / pr.count, pi = (int)blockIdx.z - ent * pr.count;
+  A += (long long)ent * sA + (long long)pi * pr.step;
+  B += (long long)ent * sB + (long long)pi * pr.step;
+  C += (long long)ent * sC + (long long)pi * pr.step;
+  if (pr.ragged) {
+    const int left = pr.rows - pi * pr.rows_step;
+    if (pr.ragged == 1) {
+      M = min(M, left);
+      K = min(K, left);
+    } else {
+      N = min(N, left);
+    }
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int i0 = blockIdx.y * kT3BM, j0 = blockIdx.x * kT3BN;
-  if (lower && j0 > i0 + kT3BM - 1) return;
+  if ((lower && j0 > i0 + kT3BM - 1) || i0 >= M || j0 >= N) return;
+  if (kdiag == 4) K = min(K, i0 + kT3BM);
   const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;   // the warp's 32 x 32 quarter
   const int g = lane >> 2, t = lane & 3;                    // mma group and thread in group
   float acc[2][4][4];
@@ -74,7 +98,7 @@ k_gemm_tf32x3(int M, int N, int K, const float* __restrict__ A, int lda, long lo
     for (int b = 0; b < 4; ++b)
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-  const int kfirst = kdiag == 2 ? max(i0, j0) : (kdiag == 1 ? j0 : 0);
+  const int kfirst = kdiag == 2 ? max(i0, j0) : (kdiag == 1 ? j0 : (kdiag == 3 ? i0 : 0));
   constexpr int kPer = kT3BM * kT3BK / kT3Threads;   // tile elements per thread and operand (16)
   float ra[kPer], rb[kPer];
   // loads run along each operand's contiguous dimension
@@ -173,11 +197,15 @@ k_gemm_tf32x3(int M, int N, int K, const float* __restrict__ A, int lda, long lo
 template <bool TA, bool TB>
 inline void gemm_tf32x3(cudaStream_t st, int M, int N, int K, const float* A, int lda, const float* B, int ldb,
                         float* C, int ldc, float alpha = 1.f, float beta = 0.f, int batch = 1, long long sA = 0,
-                        long long sB = 0, long long sC = 0, bool lower = false, int kdiag = 0) {
+                        long long sB = 0, long long sC = 0, bool lower = false, int kdiag = 0,
+                        const T3Pairs& pr = T3Pairs()) {
   if (M <= 0 || N <= 0) return;
-  dim3 grid((N + kT3BN - 1) / kT3BN, (M + kT3BM - 1) / kT3BM, batch);
-  k_gemm_tf32x3<TA, TB><<<grid, kT3Threads, 0, st>>>(M, N, K, A, lda, sA, B, ldb, sB, C, ldc, sC, alpha, beta,
-                                                     lower ? 1 : 0, kdiag);
+  const int most = 65535 / pr.count;   // entries a launch (the grid's z extent)
+  for (int b0 = 0; b0 < batch; b0 += most) {
+    dim3 grid((N + kT3BN - 1) / kT3BN, (M + kT3BM - 1) / kT3BM, std::min(most, batch - b0) * pr.count);
+    k_gemm_tf32x3<TA, TB><<<grid, kT3Threads, 0, st>>>(M, N, K, A + b0 * sA, lda, sA, B + b0 * sB, ldb, sB,
+                                                       C + b0 * sC, ldc, sC, alpha, beta, lower ? 1 : 0, kdiag, pr);
+  }
 }
 
 }  // namespace

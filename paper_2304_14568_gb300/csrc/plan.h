@@ -109,11 +109,13 @@ struct Plan {
   Ctl *ctl = nullptr;             // device control block
   Ctl *ctl_host = nullptr;        // pinned mirror
 
-  // cached-factor subproblem (chol.cu): B_s^{-1} [N][n][n] FP32, A~_s^T p~ [N][n],
+  // cached-factor subproblem (chol.cu): B_s^{-1} [N][n][chol_ld(n)] FP32, the
+  // workspace L^{-1} of the same size (allocated with it), A~_s^T p~ [N][n],
   // record index of kept row k in scenario s's list [N][m_act] (-1: empty there)
-  float *binv = nullptr;
+  float *binv = nullptr, *chol_y = nullptr;
   double *bchol = nullptr;
   int *rec_of = nullptr;
+  double *reweight = nullptr;      // workspace of rpt_plan_set_weights (allocated on its first call)
   double *trace = nullptr;         // [kTraceCap][kTraceFields] (allocated on first traced solve)
   int trace_count = 0;             // entries of the last traced solve
   bool chol_ready = false;
@@ -157,9 +159,12 @@ struct Plan {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 };
 
+// Leading dimension of B_s and its inverse: rows start on 16 bytes.
+inline __host__ __device__ int chol_ld(int n) { return (n + 3) & ~3; }
+
 // chol.cu: form, factor and invert B_s for this rho; `extra` (may be null) adds
 // further terms to the lower triangle of every B_s before the factorisation
-// (B_s row-major [N][n][n] float, launched on the plan's stream) and marks the
+// (B_s row-major [N][n][chol_ld(n)] float, launched on the plan's stream) and marks the
 // factor as not reusable by plain solves
 struct CholExtra {
   virtual cudaError_t add(Plan* P, float* B) = 0;

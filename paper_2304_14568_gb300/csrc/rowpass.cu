@@ -619,10 +619,12 @@ cudaError_t bundle_bounds_t(const DevPlan& P, double* kc, double* pc, double* kb
 }
 
 // ---- reweighting (rpt_plan_set_weights) ------------------------------------
-// Row records of scenario s for new weights: c_s w_k and p_k of every listed row
+// Row records of every scenario (grid.y) for new weights: c_s w_k and p_k of every listed row
 // (kept index k), as float32 bits like plan creation writes them.
-__global__ void k_reweight_rows(DevPlan P, int s, double cs, const double* __restrict__ wk,
+__global__ void k_reweight_rows(DevPlan P, const double* __restrict__ csv, const double* __restrict__ wk,
                                 const double* __restrict__ pk) {
+  const int s = blockIdx.y;
+  const double cs = csv[s];
   int4* rec = const_cast<int4*>(P.rowrec) + P.rec_base[s];
   const int span = P.rec_base[s + 1] - P.rec_base[s];
   const int stride = gridDim.x * blockDim.x;
@@ -644,12 +646,15 @@ __global__ void k_reweight_rows(DevPlan P, int s, double cs, const double* __res
   }
 }
 
-// Jacobi diagonal of scenario s, sum_i c_s w_i a_ij^2, as exact 64-bit fixed-point
-// sums (scale 2^F given by the caller from a bound), one warp per row or bundle;
+// Jacobi diagonal of every scenario (grid.y), sum_i c_s w_i a_ij^2, as exact 64-bit
+// fixed-point sums (scales 2^F given by the caller from bounds), one warp per row or bundle;
 // a = the stored value (dequantised).
 template <typename VT, typename IT>
-__global__ void k_reweight_diag(DevPlan P, int s, double cs, const double* __restrict__ wk, double scale,
-                                unsigned long long* __restrict__ acc) {
+__global__ void k_reweight_diag(DevPlan P, const double* __restrict__ csv, const double* __restrict__ wk,
+                                const double* __restrict__ scv, unsigned long long* __restrict__ accv) {
+  const int s = blockIdx.y;
+  const double cs = csv[s], scale = scv[s];
+  unsigned long long* acc = accv + (size_t)s * P.n_pad;
   const int lane = threadIdx.x & 31;
   const int4* rec = P.rowrec + P.rec_base[s];
   const int span = P.rec_base[s + 1] - P.rec_base[s];
@@ -693,30 +698,30 @@ __global__ void k_reweight_diag(DevPlan P, int s, double cs, const double* __res
 }
 
 template <typename VT, typename IT>
-cudaError_t reweight_t(const DevPlan& P, int s, double cs, const double* wk, const double* pk, double scale,
-                       unsigned long long* acc, cudaStream_t st) {
-  k_reweight_rows<<<P.grid, 256, 0, st>>>(P, s, cs, wk, pk);
-  cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * P.n_pad, st);
+cudaError_t reweight_t(const DevPlan& P, const double* cs, const double* wk, const double* pk, const double* scale,
+                       unsigned long long* acc, int blocks, cudaStream_t st) {
+  k_reweight_rows<<<dim3(blocks, P.N), 256, 0, st>>>(P, cs, wk, pk);
+  cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * (size_t)P.N * P.n_pad, st);
   if (e != cudaSuccess) return e;
-  k_reweight_diag<VT, IT><<<P.grid, 256, 0, st>>>(P, s, cs, wk, scale, acc);
+  k_reweight_diag<VT, IT><<<dim3(blocks, P.N), 256, 0, st>>>(P, cs, wk, scale, acc);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t plan_reweight(const DevPlan& P, int s, double cs, const double* wk, const double* pk, double scale,
-                          unsigned long long* acc, cudaStream_t st) {
+cudaError_t plan_reweight(const DevPlan& P, const double* cs, const double* wk, const double* pk,
+                          const double* scale, unsigned long long* acc, int blocks, cudaStream_t st) {
   if (P.index_width == 16) {
     switch (P.value_format) {
-      case 1: return reweight_t<__nv_bfloat16, uint16_t>(P, s, cs, wk, pk, scale, acc, st);
-      case 2: return reweight_t<__nv_fp8_e4m3, uint16_t>(P, s, cs, wk, pk, scale, acc, st);
-      default: return reweight_t<float, uint16_t>(P, s, cs, wk, pk, scale, acc, st);
+      case 1: return reweight_t<__nv_bfloat16, uint16_t>(P, cs, wk, pk, scale, acc, blocks, st);
+      case 2: return reweight_t<__nv_fp8_e4m3, uint16_t>(P, cs, wk, pk, scale, acc, blocks, st);
+      default: return reweight_t<float, uint16_t>(P, cs, wk, pk, scale, acc, blocks, st);
     }
   }
   switch (P.value_format) {
-    case 1: return reweight_t<__nv_bfloat16, int32_t>(P, s, cs, wk, pk, scale, acc, st);
-    case 2: return reweight_t<__nv_fp8_e4m3, int32_t>(P, s, cs, wk, pk, scale, acc, st);
-    default: return reweight_t<float, int32_t>(P, s, cs, wk, pk, scale, acc, st);
+    case 1: return reweight_t<__nv_bfloat16, int32_t>(P, cs, wk, pk, scale, acc, blocks, st);
+    case 2: return reweight_t<__nv_fp8_e4m3, int32_t>(P, cs, wk, pk, scale, acc, blocks, st);
+    default: return reweight_t<float, int32_t>(P, cs, wk, pk, scale, acc, blocks, st);
   }
 }
 

@@ -870,49 +870,49 @@ __global__ void k_chol_rhs(DevPlan P, const Ctl* __restrict__ C, const double* _
 }
 
 // Cached-factor x-update, part 2 (App. A): x_s = B_s^{-1} c_s.  grid (ceil(n /
-// kCholRows), N), 256 threads: c_s staged in shared memory, each warp takes rows
-// of B_s^{-1} (streamed once, evict-first) with four 16-byte loads in flight per
-// lane, FP64 accumulation of FP32 products.
+// rows), N), 256 threads: c_s staged in shared memory, each warp takes rows of
+// B_s^{-1} (16-byte aligned, zero beyond column n) with four 16-byte loads in
+// flight per lane, FP64 accumulation of FP32 products.  rows (chol_rows) keeps at
+// least four CTAs per SM on small plans.
 constexpr int kCholRows = 64;
+inline int chol_rows(int n, int N, int sms) {
+  int rows = kCholRows;
+  while (rows > 8 && (long long)((n + rows - 1) / rows) * N < 4ll * sms) rows /= 2;
+  return rows;
+}
 __global__ void __launch_bounds__(256)
 k_chol_x(DevPlan P, const Ctl* __restrict__ C, const float* __restrict__ binv, const float* __restrict__ c,
-         double* x) {
+         double* x, int rows) {
   extern __shared__ float cbuf[];
-  const int s = blockIdx.y, n = P.n;
+  const int s = blockIdx.y, n = P.n, ld = chol_ld(n);
   if (C->g[s / P.Ns].done) return;   // a stopped group keeps its x
-  for (int j = threadIdx.x; j < n; j += blockDim.x) cbuf[j] = c[(size_t)s * P.n_pad + j];
+  for (int j = threadIdx.x; j < ld; j += blockDim.x) cbuf[j] = j < n ? c[(size_t)s * P.n_pad + j] : 0.f;
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const float* Bs = binv + (size_t)s * n * n;
-  const bool vec = (n & 3) == 0;
-  for (int r = w; r < kCholRows; r += 8) {
-    const int j = blockIdx.x * kCholRows + r;
+  const float* Bs = binv + (size_t)s * n * ld;
+  const float4* c4 = reinterpret_cast<const float4*>(cbuf);
+  const int nq = ld >> 2;
+  for (int r = w; r < rows; r += 8) {
+    const int j = blockIdx.x * rows + r;
     if (j >= n) break;
-    const float* row = Bs + (size_t)j * n;
+    const float4* row4 = reinterpret_cast<const float4*>(Bs + (size_t)j * ld);
     double acc = 0.0;
-    if (vec) {
-      const float4* row4 = reinterpret_cast<const float4*>(row);
-      const float4* c4 = reinterpret_cast<const float4*>(cbuf);
-      const int nq = n >> 2;
-      int k = lane;
-      for (; k + 96 < nq; k += 128) {
-        const float4 b0 = __ldcs(row4 + k), b1 = __ldcs(row4 + k + 32), b2 = __ldcs(row4 + k + 64),
-                     b3 = __ldcs(row4 + k + 96);
-        const float4 v0 = c4[k], v1 = c4[k + 32], v2 = c4[k + 64], v3 = c4[k + 96];
-        float t = b0.x * v0.x + b0.y * v0.y + b0.z * v0.z + b0.w * v0.w;
-        t += b1.x * v1.x + b1.y * v1.y + b1.z * v1.z + b1.w * v1.w;
-        acc += (double)t;
-        t = b2.x * v2.x + b2.y * v2.y + b2.z * v2.z + b2.w * v2.w;
-        t += b3.x * v3.x + b3.y * v3.y + b3.z * v3.z + b3.w * v3.w;
-        acc += (double)t;
-      }
-      for (; k < nq; k += 32) {
-        const float4 b = __ldcs(row4 + k);
-        const float4 v = c4[k];
-        acc += (double)(b.x * v.x + b.y * v.y + b.z * v.z + b.w * v.w);
-      }
-    } else {
-      for (int k = lane; k < n; k += 32) acc += (double)(__ldcs(row + k) * cbuf[k]);
+    int k = lane;
+    for (; k + 96 < nq; k += 128) {
+      const float4 b0 = __ldcs(row4 + k), b1 = __ldcs(row4 + k + 32), b2 = __ldcs(row4 + k + 64),
+                   b3 = __ldcs(row4 + k + 96);
+      const float4 v0 = c4[k], v1 = c4[k + 32], v2 = c4[k + 64], v3 = c4[k + 96];
+      float t = b0.x * v0.x + b0.y * v0.y + b0.z * v0.z + b0.w * v0.w;
+      t += b1.x * v1.x + b1.y * v1.y + b1.z * v1.z + b1.w * v1.w;
+      acc += (double)t;
+      t = b2.x * v2.x + b2.y * v2.y + b2.z * v2.z + b2.w * v2.w;
+      t += b3.x * v3.x + b3.y * v3.y + b3.z * v3.z + b3.w * v3.w;
+      acc += (double)t;
+    }
+    for (; k < nq; k += 32) {
+      const float4 b = __ldcs(row4 + k);
+      const float4 v = c4[k];
+      acc += (double)(b.x * v.x + b.y * v.y + b.z * v.z + b.w * v.w);
     }
     acc = warp_sum_d(acc);
     if (lane == 0) x[(size_t)s * n + j] = acc;
@@ -1071,12 +1071,18 @@ void admm_tail_final(Exec& e, Plan* P) {
   launch(e, k_final_obj, dim3(1), dim3(32), 0, P->dp, P->ctl);
 }
 
+void chol_x(Exec& e, Plan* P) {
+  const DevPlan& dp = P->dp;
+  const int rows = chol_rows(dp.n, dp.N, P->sm_count);
+  launch(e, k_chol_x, dim3((dp.n + rows - 1) / rows, dp.N), dim3(256), sizeof(float) * (size_t)dp.n_pad, dp,
+         (const Ctl*)P->ctl, (const float*)P->binv, (const float*)P->v32, P->x, rows);
+}
+
 void chol_iteration_head(Exec& e, Plan* P) {
   const DevPlan& dp = P->dp;
   launch(e, k_chol_rhs, dim3(P->nchunk, dp.N), dim3(VT), 0, dp, (const Ctl*)P->ctl, (const double*)P->bchol,
          (const double*)P->z, (const double*)P->y, P->v32);
-  launch(e, k_chol_x, dim3((dp.n + kCholRows - 1) / kCholRows, dp.N), dim3(256), sizeof(float) * (size_t)dp.n_pad,
-         dp, (const Ctl*)P->ctl, (const float*)P->binv, (const float*)P->v32, P->x);
+  chol_x(e, P);
 }
 
 cudaError_t build_admm_chol_graph(Plan* P, int use_obj) {
@@ -1392,9 +1398,7 @@ int admm_solve_impl(Plan* P, const rpt_admm_params* prm, const double* z0, const
       ex.st = st;
       if (con) {
         if ((e = con->rhs(P))) return cuda_fail(e, "dose-constraint right-hand side");
-        launch(ex, k_chol_x, dim3((dp.n + kCholRows - 1) / kCholRows, dp.N), dim3(256),
-               sizeof(float) * (size_t)dp.n_pad, dp, (const Ctl*)P->ctl, (const float*)P->binv,
-               (const float*)P->v32, P->x);
+        chol_x(ex, P);
       } else {
         chol_iteration_head(ex, P);
       }

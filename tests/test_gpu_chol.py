@@ -83,3 +83,40 @@ def test_quantised_plan_uses_the_dequantised_matrix(rpt, fmt):
     with plan_of(rpt, prob, value_format=fmt, index_width=16) as P:
         z, info = P.admm_bb_solve(eps_abs=1e-6, eps_rel=1e-6, max_iter=20000, subproblem=rpt.SUB_CHOL)
     assert info["status"] == 0 and (Wq.f(z) - Wq.f(xq)) / Wq.f(xq) <= 1e-6
+
+
+@pytest.mark.parametrize("path", [1, 3])
+@pytest.mark.parametrize("n,m,mean_row", [
+    (3, 40, 2.0), (63, 300, 9.0), (64, 300, 9.0), (65, 300, 9.0), (129, 300, 9.0),   # one block, two, three
+    (257, 300, 9.0), (321, 400, 9.0), (702, 500, 9.0),    # past a panel; ragged second halves while doubling
+    (1300, 64, 200.0),                                    # more columns than a block of 16 rows holds
+    (1402, 48, 700.0),                                    # ... than four rows hold
+])
+def test_factor_at_the_edges_of_its_blocks(rpt, path, n, m, mean_row):
+    """The factor, its inverse and the products at sizes around their blocks, by
+    the error budget and the relative tolerance (1e-4) of
+    test_iterates_match_oracle_cholesky_admm (two iterations: the second starts
+    from the first one's state)."""
+    prob = random_problem(29, m=m, n=n, N=2, mean_row=mean_row, scen_weight=True, ub=6.0)
+    W = Weighted(prob)
+    rho = default_rho(W)
+    K = max_col_count(prob)
+    kappa = []
+    for s in range(prob.N):
+        ev = np.linalg.eigvalsh(W.B_dense(s, rho))
+        kappa.append(ev[-1] / ev[0])
+    k = 2
+    ref = admm_bb(W, rho=rho, max_iter=k, eps_abs=0.0, eps_rel=0.0, subproblem="chol")
+    with plan_of(rpt, prob, row_path=path) as P:
+        P.admm_bb_solve(rho=rho, max_iter=k, eps_abs=0.0, eps_rel=0.0, subproblem=rpt.SUB_CHOL)
+        _, X, _ = P.state_get()
+    e2 = 0.0
+    for s in range(prob.N):
+        Aa, xs = abs(W.At[s]), np.abs(ref["x"][s])
+        cs = np.linalg.norm(W.b(s)) + 0.5 * rho * np.linalg.norm(ref["x"][s]) + np.linalg.norm(ref["y"][s])
+        e = (2.0 / rho) * EPS32 * (4.0 * prob.n * kappa[s] * cs + (K + 2) * np.linalg.norm(Aa.T @ (Aa @ xs)))
+        e2 += e * e
+    bound = 10.0 * k * math.sqrt(e2)
+    err = np.linalg.norm(X - ref["x"])
+    print(f"n {n} m {m}: error {err:.2e}, bound {bound:.2e}, norm {np.linalg.norm(ref['x']):.2e}")
+    assert err <= min(bound, 1e-4 * np.linalg.norm(ref["x"])), (err, bound)
