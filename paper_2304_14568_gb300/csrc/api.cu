@@ -172,6 +172,7 @@ void free_plan(Plan* P) {
   for (void* a : P->allocs) cudaFree(a);
   P->allocs.clear();
   if (P->ctl_host) cudaFreeHost(P->ctl_host);
+  if (P->op_host) cudaFreeHost(P->op_host);
   if (P->ev0) cudaEventDestroy(P->ev0);
   if (P->ev1) cudaEventDestroy(P->ev1);
   if (P->own_stream && P->stream) cudaStreamDestroy(P->stream);
@@ -870,10 +871,12 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
     free_plan(P);
     return cuda_fail(A.err, "device allocation");
   }
-  if ((e = cudaMallocHost(&P->ctl_host, sizeof(Ctl)))) {
+  if ((e = cudaMallocHost(&P->ctl_host, sizeof(Ctl))) ||
+      (e = cudaMallocHost(&P->op_host, sizeof(double) * (Nn + 1 + N)))) {
     free_plan(P);
     return cuda_fail(e, "pinned allocation");
   }
+  P->op_host_report = P->op_host + Nn;
   if ((e = cudaEventCreate(&P->ev0)) || (e = cudaEventCreate(&P->ev1))) {
     free_plan(P);
     return cuda_fail(e, "event");

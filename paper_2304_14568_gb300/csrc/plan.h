@@ -105,9 +105,16 @@ struct Plan {
   double *dots = nullptr;         // [N][nchunk][4]
   double *vpart = nullptr;        // [nchunk*N][8]
   double *g = nullptr, *xt = nullptr, *xp = nullptr;   // PGD [n]
-  float *dose = nullptr;          // [N][m_act] (allocated on demand)
+  // doses (allocated on demand): the pass's [N][m_act], the caller's [N][m], and the
+  // kept index of every voxel [m] (-1: none)
+  float *dose = nullptr;
+  double *dose_full = nullptr;
+  int *dose_kept = nullptr;
   Ctl *ctl = nullptr;             // device control block
   Ctl *ctl_host = nullptr;        // pinned mirror
+  // pinned, used by the operators' kernels directly: vectors in and out [N][n], then
+  // the error word and the scenarios' objectives [1 + N]
+  double *op_host = nullptr, *op_host_report = nullptr;
 
   // cached-factor subproblem (chol.cu): B_s^{-1} [N][n][chol_ld(n)] FP32, the
   // workspace L^{-1} of the same size (allocated with it), A~_s^T p~ [N][n],

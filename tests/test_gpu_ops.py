@@ -273,3 +273,39 @@ def test_set_weights_matches_a_fresh_plan(rpt, path):
             assert np.all(np.abs(Up[s] - Uq[s]) <= 2 * k * mag + 1e-300)
     xs = lsq_box(W2)
     assert (W2.f(zp) - W2.f(xs)) / W2.f(xs) <= 1e-6
+
+
+@pytest.mark.parametrize("n,m", [(1, 3), (255, 513), (256, 256), (257, 1025)])
+def test_operator_inputs_and_outputs_at_block_edges(rpt, n, m):
+    """The caller's vectors and doses at the edges of the blocks that move them:
+    the last entry of a vector is checked (the refused call changes no result and
+    no output), and the last voxel's dose arrives.  Tolerance as above."""
+    prob = random_problem(31, m=m, n=n, N=3, mean_row=min(6.0, float(n)), empty_frac=0.3)
+    W, k = Weighted(prob), fp32_op_bound(prob)
+    Wa = _abs_W(W)
+    x = np.random.default_rng(5).uniform(0.1, 2.0, size=n)
+    V = np.tile(x, (prob.N, 1))
+    with plan_of(rpt, prob) as P:
+        f, D = P.objective(x, dose=True)
+        for bad in (np.inf, -np.inf, np.nan):
+            xb, Vb = x.copy(), V.copy()
+            xb[-1] = Vb[-1, -1] = bad
+            for call in (lambda: P.objective(xb, dose=True), lambda: P.gradient(xb), lambda: P.apply_normal(Vb)):
+                with pytest.raises(Exception, match="non-finite"):
+                    call()
+        f2, D2 = P.objective(x, dose=True)
+        U = P.apply_normal(V)
+        g, f3 = P.gradient(x)
+    mag_g, fmag = np.zeros(n), 0.0
+    for s in range(prob.N):
+        ax = Wa.At[s] @ x + Wa.pt[s]
+        fmag += float(np.sum(ax ** 2))
+        mag_g += 2.0 * (Wa.At[s].T @ ax)
+        assert np.all(np.abs(D[s] - W.dose(s, x)) <= k * (abs(W.A[s]) @ x) + 1e-300)
+        mag = Wa.At[s].T @ (Wa.At[s] @ x)
+        assert np.all(np.abs(U[s] - W.normal_apply(s, x, 0.0)) <= k * mag + fixed_point_slack(prob, s, x) + 1e-300)
+    slack = sum(2.0 * fixed_point_slack(prob, s, x, resid=True) for s in range(prob.N))
+    assert np.all(np.abs(g - W.grad(x)) <= k * mag_g + slack + 1e-300)
+    np.testing.assert_array_equal(D2, D)
+    for v in (f, f2, f3):
+        assert abs(v - W.f(x)) <= 2 * k * fmag
