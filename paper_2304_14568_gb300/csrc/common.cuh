@@ -123,26 +123,29 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// Block-wide sum of K doubles per thread; result valid in thread 0.
+// Block-wide sums of K doubles per thread; results valid in warp 0.  Warp 0 adds the
+// warps' values lane by lane (four chains, warps c, c + 4, ...), then across its lanes:
+// (warps + 5) K double additions a block instead of 5 (warps + 1) K with a butterfly
+// in every warp, on a pipe that takes two lanes a cycle.  Warps that are not launched
+// count as zeros.
 template <int K>
-__device__ __forceinline__ void block_sum_d(double (&v)[K], double* sh /* [K*32] */) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < K; ++k) v[k] = warp_sum_d(v[k]);
+__device__ __forceinline__ void block_sum_d(double (&v)[K], double* sh /* [K * blockDim.x] */) {
+  const int nt = blockDim.x, lane = threadIdx.x & 31;
   __syncthreads();
-  if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < K; ++k) sh[k * 32 + wid] = v[k];
+  for (int k = 0; k < K; ++k) sh[k * nt + threadIdx.x] = v[k];
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const double* p = sh + k * nt + lane;
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int w = 0; w < nt; w += 128)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (w + 32 * c < nt) t[c] += p[w + 32 * c];
+    v[k] = warp_sum_d((t[0] + t[1]) + (t[2] + t[3]));
   }
-  __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      double t = lane < nw ? sh[k * 32 + lane] : 0.0;
-      v[k] = warp_sum_d(t);
-    }
-  }
-  __syncthreads();
 }
 
 // Error-free transformation: s + e == a + b exactly (Knuth's two-sum).

@@ -53,7 +53,7 @@ __global__ void k_bias_grad(int M, int N, const float* __restrict__ dH, float* _
 __global__ void k_mse(int rows, int cols, const float* __restrict__ out, const float* __restrict__ y,
                       float* __restrict__ d, __nv_bfloat16* __restrict__ db, int ldb, double inv,
                       double* __restrict__ loss) {
-  __shared__ double sh[32];
+  __shared__ double sh[256];
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();
   const int64_t n = (int64_t)rows * cols;

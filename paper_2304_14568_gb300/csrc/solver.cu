@@ -128,7 +128,7 @@ __device__ __forceinline__ bool last_block(unsigned int* counter, unsigned int t
 // (a fixed order for a given launch shape).  Result valid in thread 0.
 template <int K>
 __device__ __forceinline__ void last_block_sums(const double* buf, int count, int stride, int off, double (&S)[K],
-                                                double* sh /* [K*32] */) {
+                                                double* sh /* [K * blockDim.x] */) {
 #pragma unroll
   for (int k = 0; k < K; ++k) S[k] = 0.0;
   for (int b = threadIdx.x; b < count; b += blockDim.x)
@@ -209,17 +209,21 @@ __global__ void k_cg_init(DevPlan P, Ctl* C, const float* __restrict__ partial,
                           double* u, float* v32, double* dots, int nchunk, double* gam, double* tol,
                           double* r0n, int* act, int* cgi, unsigned int* cnt_s, unsigned long long hcg,
                           int use_cond) {
-  __shared__ double sh[2 * 32];
+  __shared__ double sh[2 * VT];
   const int s = blockIdx.y, gi = s / P.Ns, j = blockIdx.x * VT + threadIdx.x;
   const Grp& G = C->g[gi];
   const bool live = !G.done;
   const double rho = G.rho;
   double v[2] = {0.0, 0.0};
-  if (live && j < P.n) {
-    const size_t o = (size_t)s * P.n + j;
+  // (a stopped group's vectors are read too: the loads don't wait for its flag)
+  const bool in = j < P.n;
+  const size_t o = (size_t)s * P.n + j;
+  const double xj = in ? x[o] : 0.0, zj = in ? z[(size_t)gi * P.n + j] : 0.0, yj = in ? y[o] : 0.0;
+  const double mj = in ? dinv[o] : 0.0;
+  if (live && in) {
     const double gj = sum_partials(P, partial, s, j);
-    const double ri = -gj - 0.5 * rho * (x[o] - z[(size_t)gi * P.n + j]) - 0.5 * y[o];
-    const double ui = dinv[o] * ri;
+    const double ri = -gj - 0.5 * rho * (xj - zj) - 0.5 * yj;
+    const double ui = mj * ri;
     r[o] = ri;
     u[o] = ui;
     v32[(size_t)s * P.n_pad + j] = (float)ui;
@@ -289,9 +293,13 @@ __global__ void k_cg_init(DevPlan P, Ctl* C, const float* __restrict__ partial,
 // one counter).  The scenario's scalars and slots are loaded together; every CTA
 // sends its part of a sum to the shared memory that reads it, so a barrier is
 // followed by local loads only; the counter that finds the last scenario to finish
-// also adds up how many go on.  A CG step with its pass, the rest of an iteration
-// included: 250 spots, 13 scenarios 36 us before and 28 us after; 52 units of 250
-// to 550 spots 150 us before and 112 us after.
+// also adds up how many go on; the scalars that don't wait for delta are divided by
+// a second warp while the first adds delta up; the counters are loaded with the rest.
+// Double additions are slow here (two lanes a cycle), hence block_sum_d's form.  The
+// kernel at 250 spots and 13 scenarios: 11.2 us (13.1 with a butterfly in every warp
+// and each scalar loaded where it is used); a CG step with its pass, the rest of an
+// iteration included: 36 us at first, 28 with the first four of these, 26 with all;
+// 52 units of 250 to 550 spots 150 us at first, 109 with all.
 constexpr int kCgCluster = 8;
 constexpr int kCgSub = 4;
 constexpr int kCgThreads = kCgSub * kVecThreads;
@@ -311,9 +319,9 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
           const float* __restrict__ partial, const double* __restrict__ dinv, float* v32, double* gam,
           double* gprev, double* aprev, const double* __restrict__ tol, int* act, int* cgi,
           int* cgcnt, unsigned long long hcg, int use_cond) {
-  __shared__ double sh[2 * 32];
+  __shared__ double sh[2 * kCgThreads];
   __shared__ double part1[kCgCluster], part2[2 * kCgCluster];   // the cluster's parts of delta; of gamma and ||r||^2
-  __shared__ double ab[2];
+  __shared__ double ab[2], pre[2];
   cg::cluster_group cl = cg::this_cluster();
   const int nr = (int)gridDim.x;
   if ((int)cl.num_blocks() != nr) {   // never expected: report it and touch nothing
@@ -326,15 +334,25 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
   // after every CTA of the cluster has passed both barriers
   const int active = __ldcg(&act[s]);
   const int any = __ldcg(&C->cg_any);
-  const bool first = __ldcg(&cgi[s]) == 0;
+  const int steps_done = __ldcg(&cgi[s]), kcg = __ldcg(&C->kcg), cg_max = C->cg_max;
+  const bool first = steps_done == 0;
   const double hr = 0.5 * C->g[s / P.Ns].rho;
   const Slots slots = slots_of(P, s);
   double g_s = 0.0, gp_s = 0.0, ap_s = 0.0, tol_s = 0.0;
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 || threadIdx.x == 32) {
     g_s = __ldcg(&gam[s]);
     gp_s = __ldcg(&gprev[s]);
     ap_s = __ldcg(&aprev[s]);
     tol_s = __ldcg(&tol[s]);
+  }
+  // (the counters are written by the step's last scenario only, after all have come here)
+  int cnt_s = 0;
+  long long total = 0, steps = 0, passes = 0;
+  if (threadIdx.x == 0) {
+    cnt_s = __ldcg(&cgcnt[s]);
+    total = __ldcg(&C->cg_total);
+    steps = __ldcg(&C->cg_steps);
+    passes = __ldcg(&C->passes);
   }
   // the operands of the first round are loaded now, so that their latency
   // overlaps the first half's sums and barriers
@@ -350,7 +368,7 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
     x0 = x[o0];
   }
   // the same answer in every CTA of the cluster (the loop is over: a further step of the loop body)
-  if (active == 0 || any == 0 || __ldcg(&C->kcg) >= C->cg_max) return;
+  if (active == 0 || any == 0 || kcg >= cg_max) return;
   double uv[kCgChunks], wv[kCgChunks];
   double dl[1] = {0.0};
 #pragma unroll
@@ -365,13 +383,18 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
     }
   }
   block_sum_d<1>(dl, sh);
+  if (threadIdx.x == 32) {   // the scalars that don't wait for delta, while warp 0 adds it up
+    const double b = first ? 0.0 : g_s / gp_s;
+    pre[0] = b;
+    pre[1] = first ? 0.0 : b * g_s / ap_s;
+  }
   if ((int)threadIdx.x < nr) *cl.map_shared_rank(&part1[rank], (int)threadIdx.x) = dl[0];   // (valid in warp 0)
   cl.sync();
   if (threadIdx.x == 0) {
     double delta = 0.0;
     for (int k = 0; k < nr; ++k) delta += part1[k];
-    const double b = first ? 0.0 : g_s / gp_s;
-    const double den = first ? delta : delta - b * g_s / ap_s;
+    const double b = pre[0];
+    const double den = first ? delta : delta - pre[1];
     ab[0] = (den > 0.0 && isfinite(den) && isfinite(b)) ? g_s / den : 0.0;
     ab[1] = b;
   }
@@ -410,8 +433,8 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
   gprev[s] = g_s;
   aprev[s] = a;
   gam[s] = g;
-  cgi[s] += 1;
-  cgcnt[s] += 1;
+  cgi[s] = steps_done + 1;
+  cgcnt[s] = cnt_s + 1;
   act[s] = next;
   atomicAdd(reinterpret_cast<unsigned long long*>(&C->g[s / P.Ns].cg), 1ull);
   // the last of the step's `any` scenarios ends it: low half the scenarios done,
@@ -420,12 +443,12 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
   if ((int)(done & 0xffffffffull) + 1 != any) return;
   const int na = (int)(done >> 32) + next;
   C->cnt_cg = 0ull;
-  C->cg_total += any;
+  C->cg_total = total + any;
   C->cg_any = na;
-  C->kcg += 1;
-  C->cg_steps += 1;
-  C->passes += 1;
-  set_cond(hcg, use_cond, na > 0 && C->kcg < C->cg_max);
+  C->kcg = kcg + 1;
+  C->cg_steps = steps + 1;
+  C->passes = passes + 1;
+  set_cond(hcg, use_cond, na > 0 && kcg + 1 < cg_max);
 }
 
 // grid (nchunk, G).  Per group: z_new = P_box(mean_s(x_s + y_s/rho)) [std] or
@@ -433,23 +456,38 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
 __global__ void k_admm_z(DevPlan P, Ctl* C, const double* __restrict__ x, const double* __restrict__ y,
                          const double* __restrict__ z, double* znew, const double* __restrict__ lb,
                          const double* __restrict__ ub, double* vpart, int nchunk) {
-  __shared__ double sh[2 * 32];
+  __shared__ double sh[2 * VT];
   const int gi = blockIdx.y, j = blockIdx.x * VT + threadIdx.x;
   double v[2] = {0.0, 0.0};
-  if (!C->g[gi].done && j < P.n) {
+  const bool live = !C->g[gi].done;
+  if (j < P.n) {   // (a stopped group's vectors are read too: the loads don't wait for its flag)
     const double ir = C->g[gi].inv_rho;
     const bool std_form = (C->z_mode == 0);
     const size_t zo = (size_t)gi * P.n + j;
+    const double zj = z[zo], lo = lb[zo], hi = ub[zo];
     double acc = 0.0;
-    for (int s = gi * P.Ns; s < (gi + 1) * P.Ns; ++s) {
-      const size_t o = (size_t)s * P.n + j;
-      acc += std_form ? fma(y[o], ir, x[o]) : x[o];
+    const int end = (gi + 1) * P.Ns;
+    for (int s = gi * P.Ns; s < end; s += 8) {   // the loads of eight scenarios in flight, added in order
+      double a[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        a[k] = 0.0;
+        if (s + k < end) {
+          const size_t o = (size_t)(s + k) * P.n + j;
+          a[k] = std_form ? fma(y[o], ir, x[o]) : x[o];
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (s + k < end) acc += a[k];
     }
-    const double zn = clampd(acc / (double)P.Ns, lb[zo], ub[zo]);
-    znew[zo] = zn;
-    const double dz = zn - z[zo];
-    v[0] = zn * zn;
-    v[1] = dz * dz;
+    if (live) {
+      const double zn = clampd(acc / (double)P.Ns, lo, hi);
+      znew[zo] = zn;
+      const double dz = zn - zj;
+      v[0] = zn * zn;
+      v[1] = dz * dz;
+    }
   }
   block_sum_d<2>(v, sh);
   if (threadIdx.x == 0) {
@@ -473,29 +511,37 @@ __global__ void k_admm_z(DevPlan P, Ctl* C, const double* __restrict__ x, const 
 __global__ void k_admm_d(DevPlan P, Ctl* C, const double* __restrict__ x, const double* __restrict__ z,
                          const double* __restrict__ znew, const double* __restrict__ dprev, double* d,
                          double* vpart, int nchunk) {
-  __shared__ double sh[5 * 32];
+  __shared__ double sh[5 * VT];
   const int s = blockIdx.y, gi = s / P.Ns, j = blockIdx.x * VT + threadIdx.x;
   const int con = C->con_on;
   double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  if (!C->g[gi].done && j < P.n) {
+  const bool live = !C->g[gi].done;
+  if (j < P.n) {
     const size_t o = (size_t)s * P.n + j, zo = (size_t)gi * P.n + j;
-    const double xj = x[o];
-    const double dj = xj - znew[zo];
-    const double dp = dprev[o];
-    const double dd = dj - dp;
-    d[o] = dj;
-    v[0] = dd * dp;
-    v[1] = dd * dd;
-    v[2] = dj * dj;
-    v[3] = xj * xj;
-    if (con) {   // dual residual with the dose blocks: rho (z - z_prev) + sigma G_s'(v_s - v_s_prev)
+    const double xj = x[o], zn = znew[zo], dp = dprev[o];
+    if (live) {
+      const double dj = xj - zn;
+      const double dd = dj - dp;
+      d[o] = dj;
+      v[0] = dd * dp;
+      v[1] = dd * dd;
+      v[2] = dj * dj;
+      v[3] = xj * xj;
+    }
+    if (live && con) {   // dual residual with the dose blocks: rho (z - z_prev) + sigma G_s'(v_s - v_s_prev)
       const double rd = C->g[gi].rho * (znew[zo] - z[zo]) + C->con_q[o];
       v[4] = rd * rd;
     }
   }
-  block_sum_d<5>(v, sh);
   const size_t base = (size_t)P.G * nchunk;
   const int blk = s * nchunk + blockIdx.x;
+  if (con) {
+    block_sum_d<5>(v, sh);
+  } else {
+    double v4[4] = {v[0], v[1], v[2], v[3]};
+    block_sum_d<4>(v4, sh);
+    for (int k = 0; k < 4; ++k) v[k] = v4[k];
+  }
   if (threadIdx.x == 0) {
     for (int k = 0; k < 4; ++k) vpart[(base + blk) * 8 + k] = v[k];
     vpart[(base + blk) * 8 + 5] = v[4];
@@ -505,10 +551,20 @@ __global__ void k_admm_d(DevPlan P, Ctl* C, const double* __restrict__ x, const 
   for (int g = 0; g < P.G; ++g) {
     Grp& G = C->g[g];
     if (G.done) continue;   // the same for every thread of the block
-    double S[4], SC[1];
+    double S[4], SC[1] = {0.0};
     last_block_sums<4>(vpart + (base + (size_t)g * per_group) * 8, per_group, 8, 0, S, sh);
-    last_block_sums<1>(vpart + (base + (size_t)g * per_group) * 8, per_group, 8, 5, SC, sh);
+    if (con) last_block_sums<1>(vpart + (base + (size_t)g * per_group) * 8, per_group, 8, 5, SC, sh);
     const double rho = G.rho;
+    // the square roots of Eq. 9, one a lane of warp 0 (one after another in thread 0 they
+    // took a tenth of the kernel)
+    double rt = 0.0;
+    if (threadIdx.x < 32)
+      rt = sqrt(threadIdx.x == 0 ? S[2] : threadIdx.x == 1 ? G.dz2 : threadIdx.x == 2 ? G.nn : threadIdx.x == 3 ? S[3]
+                : threadIdx.x == 4 ? G.sz2 : (double)P.Ns);
+    double root[6];
+    if (threadIdx.x < 32)
+#pragma unroll
+      for (int k = 0; k < 6; ++k) root[k] = __shfl_sync(0xffffffffu, rt, k);
     const bool use_bb = C->bb_mode != 2 && G.have_prev;
     if (C->bb_scen) {
       // Eq. 8 on scenario s's own blocks: its partial sums in chunk order, and
@@ -545,7 +601,7 @@ __global__ void k_admm_d(DevPlan P, Ctl* C, const double* __restrict__ x, const 
           if (C->bb_mode == 1) step = fmin(fmax(step, rho / C->bb_kappa), C->bb_kappa * rho);
         }
       }
-      const double sN = sqrt((double)P.Ns);
+      const double sN = root[5];
       G.step = step;
       if (con) {
         // Eq. 9 extended to both blocks: r_prim over [x_s - z; G_s x_s - v_s],
@@ -556,9 +612,9 @@ __global__ void k_admm_d(DevPlan P, Ctl* C, const double* __restrict__ x, const 
         G.eps_prim = C->eps_abs * sqrt(G.nn + C->con_K) +
                      C->eps_rel * fmax(sqrt(S[3] + cs[1]), sqrt((double)P.Ns * G.sz2 + cs[2]));
       } else {
-        G.r_prim = sqrt(S[2]);
-        G.r_dual = sN * rho * sqrt(G.dz2);
-        G.eps_prim = C->eps_abs * sqrt(G.nn) + C->eps_rel * fmax(sqrt(S[3]), sN * sqrt(G.sz2));
+        G.r_prim = root[0];
+        G.r_dual = sN * rho * root[1];
+        G.eps_prim = C->eps_abs * root[2] + C->eps_rel * fmax(root[3], sN * root[4]);
       }
     }
     __syncthreads();
@@ -573,24 +629,25 @@ __global__ void k_admm_y(DevPlan P, Ctl* C, const double* __restrict__ x, double
                          const double* __restrict__ znew, const double* __restrict__ d, double* dprev,
                          float* v32, float* vz32, double* vpart, int nchunk, unsigned long long hadmm,
                          int use_cond) {
-  __shared__ double sh[32];
+  __shared__ double sh[VT];
   const int s = blockIdx.y, gi = s / P.Ns, j = blockIdx.x * VT + threadIdx.x;
   const bool live = !C->g[gi].done;
   const double step = C->bb_scen ? __ldcg(&C->step_s[s]) : __ldcg(&C->g[gi].step);
   double v[1] = {0.0};
-  if (live && j < P.n) {
-    const size_t o = (size_t)s * P.n + j, zo = (size_t)gi * P.n + j;
-    const double dj = d[o];
-    const double yn = fma(step, dj, y[o]);
+  // (a stopped group's vectors are read too: the loads don't wait for its flag)
+  const bool in = j < P.n;
+  const size_t o = (size_t)s * P.n + j, zo = (size_t)gi * P.n + j;
+  const double dj = in ? d[o] : 0.0, yj = in ? y[o] : 0.0, xj = in ? x[o] : 0.0, zj = in ? znew[zo] : 0.0;
+  if (live && in) {
+    const double yn = fma(step, dj, yj);
     y[o] = yn;
     dprev[o] = dj;
-    v32[(size_t)s * P.n_pad + j] = (float)x[o];
+    v32[(size_t)s * P.n_pad + j] = (float)xj;
     const double ye = C->con_on ? yn + C->con_t[o] : yn;   // with dose blocks: y_s + G_s' mu_s
     v[0] = ye * ye;
     if (s % P.Ns == 0) {
-      const double zn = znew[zo];
-      z[zo] = zn;
-      if (P.G == 1) vz32[j] = (float)zn;
+      z[zo] = zj;
+      if (P.G == 1) vz32[j] = (float)zj;
     }
   } else if (P.G == 1 && s == 0 && j < P.n_pad) {
     vz32[j] = 0.f;
@@ -761,7 +818,7 @@ k_pgd_grad(DevPlan P, Ctl* C, const float* __restrict__ partial,
 __global__ void k_pgd_trial(DevPlan P, Ctl* C, const double* __restrict__ x,
                             const double* __restrict__ g, const double* __restrict__ lb,
                             const double* __restrict__ ub, double* xt, float* vt32, double* vpart) {
-  __shared__ double sh[32];
+  __shared__ double sh[VT];
   const int j = blockIdx.x * VT + threadIdx.x;
   const double t = __ldcg(&C->t);
   double v[1] = {0.0};
