@@ -601,7 +601,8 @@ def main():
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "traffic_source": traffic_src or "no stored capture of this kernel variant",
-                     "kernel": ("k_rowpass_tma" if st["row_path"] in (2, 4) else "k_rowpass") +
+                     "kernel": ({4: "k_rowpass_priv (k_rowpass_tma where its accumulators don't fit)",
+                                 2: "k_rowpass_tma"}.get(st["row_path"], "k_rowpass")) +
                                f"<kNormal,f32,int32,{variant}> (CG operator pass, all scenarios)",
                      "ms_per_launch": ms_pass, "bytes_per_launch": bytes_pass,
                      "bytes_note": ("bundled layout: stored block columns (4 values + 1 index, 20 B) and 64-byte "

@@ -88,10 +88,13 @@ typedef struct {
                                        1 register-direct loads of CSR rows;
                                        2 bulk-copy (TMA) ring over CSR rows;
                                        3 streaming (warps claim chunks, entries go straight to registers);
-                                       4 bundled ring: rows grouped 4 at a time in the given row order, one
+                                       4 bundled rows: rows grouped 4 at a time in the given row order, one
                                          spot index per column of a group (rows that are neighbours in the
                                          input order should share spots, as voxels in grid order do); see
-                                         accumulate for its exact (bitwise reproducible) sums;
+                                         accumulate for its exact (bitwise reproducible) sums.  The pass
+                                         adds into private accumulators where they fit (plans of one problem
+                                         that set no ring geometry or ring_threads), else with atomics
+                                         behind a ring;
                                        0: 4 when its shared-memory stage fits the plan, else 2, else 1 */
   int32_t autotune;                 /* 1: time every ring configuration that fits this plan (entries and
                                        rows per stage, stages) on its own row pass and keep the fastest;
@@ -112,8 +115,8 @@ typedef struct {
                                        sums: every pass, and so every solve, is bitwise reproducible whatever
                                        the scheduling, and tight tolerances (1e-7) converge where float
                                        rounding noise can stall them; about 40 % slower per pass;
-                                       2 = float32 shared-memory atomics, whose results vary in the last bits
-                                       from run to run */
+                                       2 = float32 sums, whose results may vary in the last bits from run to
+                                       run (shared-memory atomics, see row_path) */
   int32_t ring_threads;             /* row path 4: threads of a row-pass CTA, 1024 (31 consumer warps, 6 block
                                        columns per lane held in registers), 768 (23 warps, 8) or 640 (19 warps,
                                        10); fewer warps hide less latency, more registers re-read fewer block

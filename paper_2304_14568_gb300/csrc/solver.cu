@@ -1823,7 +1823,7 @@ int op_objective(Plan* P, const double* x, double* f_out, double* dose_out) {
     launch(ex, k_report, dim3(1), dim3(32), 0, dp, (const int*)P->err, P->op_host_report);
   } else {
     // (the pass's doses are widened and put in the caller's order here: 0.28 ms on the
-    // host at 60,000 voxels and 13 scenarios, 5.6 MB)
+    // host at 54,000 voxels and 13 scenarios, 5.6 MB)
     const int blocks = std::max(1, std::min((dp.m + VT - 1) / VT, (4 * P->sm_count + dp.N - 1) / dp.N));
     launch(ex, k_expand_dose, dim3(blocks, dp.N), dim3(VT), 0, dp, (const int*)P->dose_kept, (const float*)P->dose,
            P->dose_full, (const int*)P->err, P->op_host_report);
