@@ -47,7 +47,7 @@ constexpr unsigned kFull = 0xffffffffu;
 // (kept-row) order; the block takes kRB / 4 consecutive bundles.
 // Bound: instruction issue (83 % of the cycles), about half of it the products of the
 // dense block and the rest the address and the atomic of each pair.  Neighbouring rows
-// share their columns, so a block of 16 rows has 0.7 of the pairs (and atomics) of two
+// share their columns, so a block of 16 rows has 0.86 of the pairs (and atomics) of two
 // blocks of 8, but its dense rows are emptier: 64 rows have half the pairs and twice
 // the products of 16.  A warp forms 8 x 64 pairs at a time from registers (16 products
 // per 4 shared loads) and takes a unit's entries with its own lanes.  A block whose
