@@ -328,10 +328,14 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
     if (threadIdx.x == 0) atomicExch(P.err, kErrCgCluster);
     return;
   }
+  // Another CTA's shared memory may be written only once that CTA has started: each
+  // says so here, and the wait stands before the first such store, behind the loads
+  // and the first half's sums.
+  auto started = cl.barrier_arrive();
   const int s = blockIdx.y, rank = (int)cl.block_rank();
   const int sub = threadIdx.x / VT, col = threadIdx.x % VT;
   // all loads in flight together; rank 0 rewrites act, cgi and the scalars only
-  // after every CTA of the cluster has passed both barriers
+  // after every CTA of the cluster has passed the last two barriers
   const int active = __ldcg(&act[s]);
   const int any = __ldcg(&C->cg_any);
   const int steps_done = __ldcg(&cgi[s]), kcg = __ldcg(&C->kcg), cg_max = C->cg_max;
@@ -368,7 +372,10 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
     x0 = x[o0];
   }
   // the same answer in every CTA of the cluster (the loop is over: a further step of the loop body)
-  if (active == 0 || any == 0 || kcg >= cg_max) return;
+  if (active == 0 || any == 0 || kcg >= cg_max) {
+    cl.barrier_wait(std::move(started));
+    return;
+  }
   double uv[kCgChunks], wv[kCgChunks];
   double dl[1] = {0.0};
 #pragma unroll
@@ -388,6 +395,7 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
     pre[0] = b;
     pre[1] = first ? 0.0 : b * g_s / ap_s;
   }
+  cl.barrier_wait(std::move(started));
   if ((int)threadIdx.x < nr) *cl.map_shared_rank(&part1[rank], (int)threadIdx.x) = dl[0];   // (valid in warp 0)
   cl.sync();
   if (threadIdx.x == 0) {
