@@ -108,7 +108,8 @@ typedef struct {
                                        power of two); 0 = 8 */
   int32_t inject_timeout;           /* testing hook: 1 makes the ring's producer (paths 2 and 4) issue no
                                        copy, so every consumer wait runs out after its one-second bound and
-                                       the call returns RPT_TIMEOUT (no GPU fault is involved); 0 normally */
+                                       the call returns RPT_TIMEOUT (no GPU fault is involved); 2 does so to
+                                       the turns on private accumulators (path 4; as 1 elsewhere); 0 normally */
   int64_t device_mem_cap;           /* testing hook: bytes the plan may allocate on the device (a request past
                                        it fails as an out-of-memory would, RPT_ENOMEM); 0 = no cap */
   int32_t accumulate;               /* row path 4's scatter: 0 = library choice (2); 1 = exact 64-bit fixed-point

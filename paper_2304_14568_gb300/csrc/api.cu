@@ -407,7 +407,7 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
   // testing hook: the bulk-copy rings' producer issues no copy, so every
   // consumer wait runs out (after its one-second bound) and the pass reports
   // RPT_TIMEOUT; the bounded waits are tested without a GPU fault
-  dp.inject_timeout = (opts && opts->inject_timeout) ? 1 : 0;
+  dp.inject_timeout = opts ? (opts->inject_timeout == 2 ? 2 : opts->inject_timeout != 0) : 0;
   dp.index_width = pr->index_width;
   P->nchunk = (n + kVecThreads - 1) / kVecThreads;
   P->kept_rows = kept;

@@ -81,7 +81,8 @@ struct DevPlan {
   const int* rec_base;                // [N+1] first record of each scenario's row list
   const ChunkDesc* chunks;            // path 1: scenario-major chunk list
   int* err;                           // device error word (bounded waits that ran out)
-  int inject_timeout;                 // testing: the ring's producer issues nothing (waits run out)
+  int inject_timeout;                 // testing: 1: the ring's producer issues nothing (waits run out); 2: the
+                                      // pass with private accumulators gives no turn (as 1 elsewhere)
   // path 3 (bundled ring): partial slots hold exact 64-bit fixed-point sums.  A
   // pass on scenario s scales every contribution by 2^fexp[s], chosen from the
   // bound |acc_c| <= kbound[2s] max|v_s| (+ kbound[2s+1] with the prescription

@@ -132,6 +132,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     if (global_ns() - t0 > kWaitLimitNs) return false;
   }
 }
+// The same for a whole warp, which goes on together: one answer for all lanes, decided by
+// votes (lanes that kept their own time could part when it runs out).
+__device__ __forceinline__ bool warp_mbar_wait(uint32_t bar, uint32_t parity) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const unsigned long long t0 = global_ns();
+  for (;;) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) return false;
+  }
+}
 // Bulk copy global -> shared; completion is counted in bytes on `bar`.
 // dst, src 16-byte aligned; bytes a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
