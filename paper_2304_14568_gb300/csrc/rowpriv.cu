@@ -86,8 +86,7 @@ __device__ __forceinline__ int ld_acquire(uint32_t addr) {
 }
 
 // Bounded wait of a whole warp for a flag in shared memory to take the value v (one
-// answer for all lanes, as warp_mbar_wait; the two votes an item cost 3 % of a BF16
-// pass at 3001 spots, 76 us, and nothing at 5000 in F32).
+// answer for all lanes, as warp_mbar_wait; the two votes an item cost no time that shows).
 __device__ __forceinline__ bool warp_flag_wait(uint32_t addr, int v) {
   if (__all_sync(kFull, ld_acquire(addr) == v)) return true;
   const unsigned long long t0 = global_ns();
@@ -104,7 +103,7 @@ struct Seg {
   float* acc;            // this warp's accumulator (float, or int64 fixed point)
   int idle;              // this lane's idle column
   float fscale;          // fixed point: 2^F
-  uint32_t turn_a;       // the accumulator's turn counter, 0: this warp has it alone
+  uint32_t turn_a;       // the accumulator's turn counter (modes that scatter)
   int turn;              // the item's turn
   bool ok;               // no wait ran out
   bool want_obj;
@@ -210,10 +209,8 @@ __device__ __forceinline__ void process_item(Seg& S, const int4* __restrict__ re
       sc[k] = cf[0] * a[k][0] + cf[1] * a[k][1] + cf[2] * a[k][2] + cf[3] * a[k][3];
       if (FIX) qv[k] = fixed_round(sc[k] * S.fscale);
     }
-    if (S.turn_a) {
-      S.ok = warp_flag_wait(S.turn_a, S.turn);
-      if (!S.ok) return;   // nothing is added out of turn, and no turn is handed on
-    }
+    S.ok = warp_flag_wait(S.turn_a, S.turn);
+    if (!S.ok) return;   // nothing is added out of turn, and no turn is handed on
     // a bundle's columns are distinct: no two lanes or slots meet
     if (kWide) {
       if (FIX) {
@@ -258,7 +255,7 @@ __device__ __forceinline__ void process_item(Seg& S, const int4* __restrict__ re
         __syncwarp();
       }
     }
-    if (S.turn_a && lane == 0) st_release(S.turn_a, S.turn + 1);
+    if (lane == 0) st_release(S.turn_a, S.turn + 1);
   }
   if (kTail) {
     __syncwarp();
@@ -511,7 +508,7 @@ k_rowpass_priv(DevPlan P, const float* __restrict__ vin, int v_stride, const int
     Seg S;
     S.sv = sv;
     S.acc = reinterpret_cast<float*>(acc0 + accs * (cw % A));
-    S.turn_a = kScatter && A < W ? smem_u32(&turns[cw % A]) : 0u;
+    S.turn_a = smem_u32(&turns[cw % A]);   // (turns are always taken: a plan has fewer accumulators than warps)
     S.ok = true;
     S.idle = P.n_pad + lane;
     S.want_obj = MODE != kNormal && objp != nullptr;

@@ -32,3 +32,9 @@ def test_a_turn_that_never_came_adds_nothing():
     wait = item.index("flag_wait(S.turn_a")
     adds = [m.start() for m in re.finditer(r"acc\[[^;]*\]\s*\+?=", item) if m.start() > wait]
     assert adds and re.search(r"if \(!S\.ok\) return;", item[wait:adds[0]])
+
+
+def test_turns_are_taken_whatever_their_address():
+    """0 is a possible address in shared memory: it cannot mean "no turns"."""
+    src = _source("rowpriv.cu")
+    assert "S.turn_a" in src and not re.search(r"\(\s*S\.turn_a\s*(\)|&&|\|\||[!=]=)|\?[^;]*turns\[[^;]*:", src)
