@@ -160,8 +160,8 @@ struct Plan {
   bool state_valid = false;
 
   // CUDA graphs (built on first use)
-  cudaGraphExec_t admm_exec = nullptr;
-  int admm_exec_obj = -1;         // use_obj flag the graph was built with
+  cudaGraphExec_t admm_exec[2] = {nullptr, nullptr};   // one, two CG steps per pass of the CG loop's body
+  int admm_exec_obj[2] = {-1, -1};                     // use_obj flag the graph was built with
   cudaGraphExec_t pgd_exec = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 };

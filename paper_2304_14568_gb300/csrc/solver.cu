@@ -437,7 +437,8 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
     g += part2[2 * k];
     rr += part2[2 * k + 1];
   }
-  const int next = (a > 0.0 && g > 0.0 && sqrt(rr) > tol_s) ? 1 : 0;
+  // (none goes on at the cap, so a further step of the loop's body finds no work)
+  const int next = (a > 0.0 && g > 0.0 && sqrt(rr) > tol_s && kcg + 1 < cg_max) ? 1 : 0;
   gprev[s] = g_s;
   aprev[s] = a;
   gam[s] = g;
@@ -456,7 +457,7 @@ k_cg_step(DevPlan P, Ctl* C, double* x, double* r, double* u, double* p, double*
   C->kcg = kcg + 1;
   C->cg_steps = steps + 1;
   C->passes = passes + 1;
-  set_cond(hcg, use_cond, na > 0 && kcg + 1 < cg_max);
+  set_cond(hcg, use_cond, na > 0);
 }
 
 // grid (nchunk, G).  Per group: z_new = P_box(mean_s(x_s + y_s/rho)) [std] or
@@ -1216,12 +1217,12 @@ cudaError_t build_admm_chol_graph(Plan* P, int use_obj) {
 // CG steps per pass of the CG loop's body: the loop node costs about 2 us a pass,
 // and a step after the last one finds no active scenario (its row pass has no
 // work).  250 spots, 30 iterations: 8.44 ms with one, 8.16 with two; realistic plan,
-// 12 iterations: 33.9 and 33.6 ms; three and four gain no more.
-constexpr int kCgUnroll = 2;
+// 12 iterations: 33.9 and 33.6 ms; three and four gain no more.  With a cap of one
+// every loop would end on such an empty step (an iteration at 250 spots 97 us against
+// 92 with one step per body; cap three 145 and 145, five 193 and 197).
+inline int cg_steps_per_body(int cg_max) { return cg_max < 2 ? 1 : 2; }
 
-cudaError_t build_admm_graph(Plan* P, int use_obj, double* z0d, double* y0d) {
-  (void)z0d;
-  (void)y0d;
+cudaError_t build_admm_graph(Plan* P, int use_obj, int steps) {
   cudaGraph_t g = nullptr;
   cudaError_t err = cudaGraphCreate(&g, 0);
   if (err != cudaSuccess) return err;
@@ -1235,17 +1236,18 @@ cudaError_t build_admm_graph(Plan* P, int use_obj, double* z0d, double* y0d) {
     body.err = cudaGraphConditionalHandleCreate(&hcg, body.g, 0, cudaGraphCondAssignDefault);
   admm_iteration_head(body, P, (unsigned long long)hcg, 1);
   Exec cg = body.while_body(hcg);
-  for (int k = 0; k < kCgUnroll; ++k) cg_body(cg, P, (unsigned long long)hcg, 1);
+  for (int k = 0; k < steps; ++k) cg_body(cg, P, (unsigned long long)hcg, 1);
   if (cg.err != cudaSuccess) body.err = cg.err;
   admm_iteration_tail(body, P, use_obj, (unsigned long long)hadmm, 1);
   if (body.err != cudaSuccess) top.err = body.err;
   admm_tail_final(top, P);
   err = top.err;
   if (err == cudaSuccess) {
-    if (P->admm_exec) cudaGraphExecDestroy(P->admm_exec);
-    P->admm_exec = nullptr;
-    err = cudaGraphInstantiate(&P->admm_exec, g, 0);
-    if (err == cudaSuccess) P->admm_exec_obj = use_obj;
+    cudaGraphExec_t& exec = P->admm_exec[steps - 1];
+    if (exec) cudaGraphExecDestroy(exec);
+    exec = nullptr;
+    err = cudaGraphInstantiate(&exec, g, 0);
+    if (err == cudaSuccess) P->admm_exec_obj[steps - 1] = use_obj;
   }
   cudaGraphDestroy(g);
   return err;
@@ -1337,10 +1339,12 @@ cudaError_t read_ctl(Plan* P) {
 // ===========================================================================
 
 void destroy_graphs(Plan* P) {
-  if (P->admm_exec) cudaGraphExecDestroy(P->admm_exec);
+  for (cudaGraphExec_t& g : P->admm_exec) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  }
   if (P->admm_chol_exec) cudaGraphExecDestroy(P->admm_chol_exec);
   if (P->pgd_exec) cudaGraphExecDestroy(P->pgd_exec);
-  P->admm_exec = nullptr;
   P->admm_chol_exec = nullptr;
   P->pgd_exec = nullptr;
 }
@@ -1520,10 +1524,11 @@ int admm_solve_impl(Plan* P, const rpt_admm_params* prm, const double* z0, const
     admm_tail_final(ex, P);
     if (ex.err) return cuda_fail(ex.err, "launch");
   } else if (prm->use_graph) {
-    if (!P->admm_exec || P->admm_exec_obj != use_obj) {
-      if ((e = build_admm_graph(P, use_obj, nullptr, nullptr))) return cuda_fail(e, "build ADMM graph");
+    const int steps = cg_steps_per_body(prm->cg_max);
+    if (!P->admm_exec[steps - 1] || P->admm_exec_obj[steps - 1] != use_obj) {
+      if ((e = build_admm_graph(P, use_obj, steps))) return cuda_fail(e, "build ADMM graph");
     }
-    if ((e = cudaGraphLaunch(P->admm_exec, st))) return cuda_fail(e, "launch ADMM graph");
+    if ((e = cudaGraphLaunch(P->admm_exec[steps - 1], st))) return cuda_fail(e, "launch ADMM graph");
   } else {
     const int every = prm->check_every > 0 ? prm->check_every : 1;
     for (;;) {
