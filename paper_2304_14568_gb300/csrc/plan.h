@@ -105,11 +105,12 @@ struct Plan {
   double *dots = nullptr;         // [N][nchunk][4]
   double *vpart = nullptr;        // [nchunk*N][8]
   double *g = nullptr, *xt = nullptr, *xp = nullptr;   // PGD [n]
-  // doses (allocated on demand): the pass's [N][m_act], the caller's [N][m], and the
-  // kept index of every voxel [m] (-1: none)
+  // doses (allocated on demand): the pass's [N][m_act], the kept index of every voxel
+  // [m] (-1: none), and the staging buffer of the caller's [N][m] (its doubles)
   float *dose = nullptr;
-  double *dose_full = nullptr;
-  int *dose_kept = nullptr;
+  int *dose_idx = nullptr;
+  double *dose_stage = nullptr;
+  size_t dose_stage_len = 0;
   Ctl *ctl = nullptr;             // device control block
   Ctl *ctl_host = nullptr;        // pinned mirror
   // pinned, used by the operators' kernels directly: vectors in and out [N][n], then

@@ -941,15 +941,22 @@ __global__ void k_reduce_scen(DevPlan P, const float* __restrict__ partial, doub
   io[o] = sum_partials(P, partial, s, j) + half_rho * v;
 }
 
-// grid (blocks, N).  The caller's dose array [N][m] from the pass's [N][m_act]:
-// kept[i] = kept index of voxel i, -1 where it has no entry.
-__global__ void k_expand_dose(DevPlan P, const int* __restrict__ kept, const float* __restrict__ dose,
-                              double* __restrict__ out, const int* err, double* report) {
-  if (blockIdx.x == 0 && blockIdx.y == 0) op_report(P, err, true, report);
-  const size_t s = blockIdx.y;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.m; i += gridDim.x * blockDim.x) {
-    const int k = kept[i];
-    out[s * P.m + i] = k >= 0 ? (double)dose[s * P.m_act + k] : 0.0;
+// idx[kept[k]] = k (idx -1 elsewhere): the kept index of every voxel.
+__global__ void k_dose_index(int m_act, const int* __restrict__ kept, int* __restrict__ idx) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m_act; k += gridDim.x * blockDim.x) idx[kept[k]] = k;
+}
+
+// grid (blocks, scenarios of the piece).  Voxels [i0, i0 + len) of scenarios s0, s0 + 1, ... of
+// the caller's dose array [N][m] from the pass's [N][m_act]: idx[i] = kept index of voxel
+// i, -1 where it has no entry.  report (may be null): the operator's report.
+__global__ void k_expand_dose(DevPlan P, const int* __restrict__ idx, const float* __restrict__ dose, int s0, int i0,
+                              int len, double* __restrict__ out, const int* err, double* report) {
+  if (report != nullptr && blockIdx.x == 0 && blockIdx.y == 0) op_report(P, err, true, report);
+  const float* from = dose + (size_t)(s0 + blockIdx.y) * P.m_act;
+  double* to = out + (size_t)blockIdx.y * len;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < len; i += gridDim.x * blockDim.x) {
+    const int k = idx[i0 + i];
+    to[i] = k >= 0 ? (double)from[k] : 0.0;
   }
 }
 
@@ -1796,29 +1803,56 @@ int op_gradient(Plan* P, const double* x, double* g_out, double* f_out) {
 }
 
 // The buffers of a dose, on the first call that asks for one: the pass's [N][m_act],
-// the caller's [N][m] and the kept index of every voxel.
+// the kept index of every voxel [m], made on the device from the list of kept rows, and
+// the staging buffer for the caller's [N][m], which large volumes take in pieces:
+// 32 MB (208 MB of doses in seven pieces: 1.28 ms a call, the copies 0.2 ms each), less
+// where memory is short.
+constexpr size_t kDoseStage = (size_t)4 << 20, kDoseStageMin = (size_t)8 << 10;   // doubles
 static int dose_buffers(Plan* P) {
   const DevPlan& dp = P->dp;
   if (P->dose) return RPT_OK;
-  const size_t act = ((size_t)dp.N * dp.m_act + 1) & ~(size_t)1, full = (size_t)dp.N * dp.m;
-  std::vector<int> kept(dp.m, -1);
-  for (int k = 0; k < dp.m_act; ++k) kept[P->kept_rows[k]] = k;
+  const size_t act = (size_t)dp.N * dp.m_act, full = (size_t)dp.N * dp.m;
   double* d = nullptr;
-  cudaError_t e = cudaMalloc(&d, sizeof(double) * full + sizeof(float) * act + sizeof(int) * (size_t)dp.m);
-  if (e != cudaSuccess) {
-    set_error("out of device memory for doses");
-    return RPT_ENOMEM;
+  size_t stage = std::min(full, kDoseStage);
+  cudaError_t e;
+  while ((e = cudaMalloc(&d, sizeof(double) * stage + sizeof(float) * act + sizeof(int) * (size_t)dp.m))) {
+    if (stage <= kDoseStageMin) {
+      set_error("out of device memory for doses");
+      return RPT_ENOMEM;
+    }
+    cudaGetLastError();
+    stage = std::max(stage / 8, kDoseStageMin);
   }
   P->allocs.push_back(d);
-  float* act_dose = reinterpret_cast<float*>(d + full);
-  int* idx = reinterpret_cast<int*>(act_dose + act);
-  if ((e = cudaMemcpyAsync(idx, kept.data(), sizeof(int) * (size_t)dp.m, cudaMemcpyHostToDevice, P->stream)) ||
-      (e = cudaStreamSynchronize(P->stream)))
+  float* dose = reinterpret_cast<float*>(d + stage);
+  int* idx = reinterpret_cast<int*>(dose + act);
+  // (the list passes through the dose array, which every call clears)
+  int* list = reinterpret_cast<int*>(dose);
+  if ((e = cudaMemsetAsync(idx, 0xff, sizeof(int) * (size_t)dp.m, P->stream)) ||
+      (e = cudaMemcpyAsync(list, P->kept_rows.data(), sizeof(int) * (size_t)dp.m_act, cudaMemcpyHostToDevice,
+                           P->stream)))
     return cuda_fail(e, "copy");
-  P->dose_full = d;
-  P->dose_kept = idx;
-  P->dose = act_dose;
+  k_dose_index<<<std::max(1, std::min(P->sm_count, (dp.m_act + VT - 1) / VT)), VT, 0, P->stream>>>(dp.m_act, list, idx);
+  if ((e = cudaGetLastError())) return cuda_fail(e, "launch");
+  P->dose_stage = d;
+  P->dose_stage_len = stage;
+  P->dose_idx = idx;
+  P->dose = dose;
   return RPT_OK;
+}
+
+// Voxels of one piece of the caller's dose array, and scenarios: whole scenarios where
+// one fits the staging buffer.
+static void dose_piece(const Plan* P, int s0, int i0, int* len, int* rows) {
+  const DevPlan& dp = P->dp;
+  *len = (int)std::min<size_t>(dp.m - i0, P->dose_stage_len);
+  *rows = *len == dp.m ? std::min(dp.N - s0, (int)std::min<size_t>(P->dose_stage_len / dp.m, 65535)) : 1;
+}
+
+static void dose_expand(Exec& ex, Plan* P, int s0, int i0, int len, int rows, double* report) {
+  const int blocks = std::max(1, std::min((len + VT - 1) / VT, (4 * P->sm_count + rows - 1) / rows));
+  launch(ex, k_expand_dose, dim3(blocks, rows), dim3(VT), 0, P->dp, (const int*)P->dose_idx, (const float*)P->dose, s0,
+         i0, len, P->dose_stage, (const int*)P->err, report);
 }
 
 int op_objective(Plan* P, const double* x, double* f_out, double* dose_out) {
@@ -1832,21 +1866,39 @@ int op_objective(Plan* P, const double* x, double* f_out, double* dose_out) {
   // rows that are empty in a scenario are not visited: their dose is zero
   if (dose_out && !ex.err) ex.err = cudaMemsetAsync(P->dose, 0, sizeof(float) * (size_t)dp.N * dp.m_act, P->stream);
   rowpass(ex, P, dose_out ? kDose : kObj, P->vz32, 0, nullptr, P->dose);
+  int s0 = 0, i0 = 0, len = 0, rows = 0;   // the piece of dose_out in the staging buffer
   if (!dose_out) {
     launch(ex, k_report, dim3(1), dim3(32), 0, dp, (const int*)P->err, P->op_host_report);
   } else {
     // (the pass's doses are widened and put in the caller's order here: 0.28 ms on the
     // host at 54,000 voxels and 13 scenarios, 5.6 MB)
-    const int blocks = std::max(1, std::min((dp.m + VT - 1) / VT, (4 * P->sm_count + dp.N - 1) / dp.N));
-    launch(ex, k_expand_dose, dim3(blocks, dp.N), dim3(VT), 0, dp, (const int*)P->dose_kept, (const float*)P->dose,
-           P->dose_full, (const int*)P->err, P->op_host_report);
+    dose_piece(P, s0, i0, &len, &rows);
+    dose_expand(ex, P, s0, i0, len, rows, P->op_host_report);
   }
+  // dose_out is written only after a pass that went well
   if (int rc = op_wait(ex, P, "launch")) return rc;
-  if (dose_out) {
-    cudaError_t e = cudaMemcpyAsync(dose_out, P->dose_full, sizeof(double) * (size_t)dp.N * dp.m,
-                                    cudaMemcpyDeviceToHost, P->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(P->stream);
-    if (e) return cuda_fail(e, "copy out");
+  while (dose_out && s0 < dp.N) {
+    cudaError_t e = cudaMemcpyAsync(dose_out + (size_t)s0 * dp.m + i0, P->dose_stage,
+                                    sizeof(double) * (size_t)rows * len, cudaMemcpyDeviceToHost, P->stream);
+    if (i0 + len < dp.m) {
+      i0 += len;
+    } else {
+      s0 += rows;
+      i0 = 0;
+    }
+    if (s0 < dp.N) {   // the next piece, behind the copy
+      dose_piece(P, s0, i0, &len, &rows);
+      if (e == cudaSuccess) {
+        dose_expand(ex, P, s0, i0, len, rows, nullptr);
+        e = ex.err;
+      }
+    } else if (e == cudaSuccess) {
+      e = cudaStreamSynchronize(P->stream);
+    }
+    if (e) {
+      cudaStreamSynchronize(P->stream);
+      return cuda_fail(e, "copy out");
+    }
   }
   if (f_out) *f_out = op_objective_value(P);
   return RPT_OK;
