@@ -1,0 +1,24 @@
+// Sum of float32 numbers carried as s + c with the rounding error of every addition
+// kept (Knuth's two-sum): as good as a float64 sum of the same numbers, in float32
+// additions, which run 64 times as fast here.  Host and device (tested on the CPU).
+#pragma once
+
+#ifdef __CUDACC__
+#define RPT_HD __host__ __device__ __forceinline__
+#else
+#define RPT_HD inline
+#endif
+
+namespace rpt {
+
+struct CompSum {
+  float s = 0.f, c = 0.f;
+  RPT_HD void add(float p) {
+    const float t = s + p, b = t - s;
+    c += (s - (t - b)) + (p - b);
+    s = t;
+  }
+  RPT_HD double value() const { return (double)s + (double)c; }
+};
+
+}  // namespace rpt

@@ -26,6 +26,7 @@
 #include <cooperative_groups.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include "compsum.h"
 #include "plan.h"
 
 namespace rpt {
@@ -981,8 +982,9 @@ __global__ void k_chol_rhs(DevPlan P, const Ctl* __restrict__ C, const double* _
 // Cached-factor x-update, part 2 (App. A): x_s = B_s^{-1} c_s.  grid (ceil(n /
 // rows), N), 256 threads: c_s staged in shared memory, each warp takes rows of
 // B_s^{-1} (16-byte aligned, zero beyond column n) with four 16-byte loads in
-// flight per lane, FP64 accumulation of FP32 products.  rows (chol_rows) keeps at
-// least four CTAs per SM on small plans.
+// flight per lane.  The products are rounded to FP32 and summed without loss
+// (CompSum, one a component: as a sum in FP64, whose pipe takes two lanes a cycle).
+// rows (chol_rows) keeps at least four CTAs per SM on small plans.
 constexpr int kCholRows = 64;
 inline int chol_rows(int n, int N, int sms) {
   int rows = kCholRows;
@@ -1005,24 +1007,24 @@ k_chol_x(DevPlan P, const Ctl* __restrict__ C, const float* __restrict__ binv, c
     const int j = blockIdx.x * rows + r;
     if (j >= n) break;
     const float4* row4 = reinterpret_cast<const float4*>(Bs + (size_t)j * ld);
-    double acc = 0.0;
+    CompSum sum[4];
+    auto add = [&](const float4& b, const float4& v) {   // (products apart: a fused one would spoil the sums' errors)
+      sum[0].add(__fmul_rn(b.x, v.x));
+      sum[1].add(__fmul_rn(b.y, v.y));
+      sum[2].add(__fmul_rn(b.z, v.z));
+      sum[3].add(__fmul_rn(b.w, v.w));
+    };
     int k = lane;
     for (; k + 96 < nq; k += 128) {
       const float4 b0 = __ldcs(row4 + k), b1 = __ldcs(row4 + k + 32), b2 = __ldcs(row4 + k + 64),
                    b3 = __ldcs(row4 + k + 96);
-      const float4 v0 = c4[k], v1 = c4[k + 32], v2 = c4[k + 64], v3 = c4[k + 96];
-      float t = b0.x * v0.x + b0.y * v0.y + b0.z * v0.z + b0.w * v0.w;
-      t += b1.x * v1.x + b1.y * v1.y + b1.z * v1.z + b1.w * v1.w;
-      acc += (double)t;
-      t = b2.x * v2.x + b2.y * v2.y + b2.z * v2.z + b2.w * v2.w;
-      t += b3.x * v3.x + b3.y * v3.y + b3.z * v3.z + b3.w * v3.w;
-      acc += (double)t;
+      add(b0, c4[k]);
+      add(b1, c4[k + 32]);
+      add(b2, c4[k + 64]);
+      add(b3, c4[k + 96]);
     }
-    for (; k < nq; k += 32) {
-      const float4 b = __ldcs(row4 + k);
-      const float4 v = c4[k];
-      acc += (double)(b.x * v.x + b.y * v.y + b.z * v.z + b.w * v.w);
-    }
+    for (; k < nq; k += 32) add(__ldcs(row4 + k), c4[k]);
+    double acc = (sum[0].value() + sum[1].value()) + (sum[2].value() + sum[3].value());
     acc = warp_sum_d(acc);
     if (lane == 0) x[(size_t)s * n + j] = acc;
   }
