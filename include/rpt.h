@@ -152,7 +152,8 @@ typedef struct {
                              operator; RPT_SUB_CHOL the cached factor: B_s = A~_s^T A~_s + (rho/2) I
                              formed, factored and inverted once per (plan, rho) in FP32 on the device,
                              then x_s = B_s^{-1} c_s each iteration (4 n^2 N bytes of device memory,
-                             plus as much again for the workspace it is formed in) */
+                             plus as much again for the workspace it is formed in, which the plan
+                             keeps if it is at most 128 MB and gives back otherwise) */
   int32_t trace;          /* 1: record one entry per iteration (see rpt_trace_get); default 0 */
   int32_t bb_per_scenario;/* 0 (default): one dual step over the concatenated vectors (Eq. 8 as
                              written); 1: Eq. 8 applied to each scenario's own blocks dd_s, dy_s,

@@ -118,7 +118,7 @@ struct Plan {
   double *op_host = nullptr, *op_host_report = nullptr;
 
   // cached-factor subproblem (chol.cu): B_s^{-1} [N][n][chol_ld(n)] FP32, the
-  // workspace L^{-1} of the same size (allocated with it), A~_s^T p~ [N][n],
+  // workspace L^{-1} of the same size (kept only while it is small), A~_s^T p~ [N][n],
   // record index of kept row k in scenario s's list [N][m_act] (-1: empty there)
   float *binv = nullptr, *chol_y = nullptr;
   double *bchol = nullptr;
