@@ -390,6 +390,22 @@ def run_scenario_sweep(args, rpt, dev, stream, prob):
 STRUCTURE_NAMES = {0: "body", 1: "target", 2: "oar1", 3: "oar2", 4: "oar3"}
 
 
+def row_pass_report(st, rp):
+    """(kernel, variant, configuration) of the row pass that a plan runs, from its stats
+    and its row_pass(); the variant keys profiles/traffic.json."""
+    sums = "exact" if st["exact_sums"] else "float"
+    if rp["accumulators"]:
+        return ("k_rowpass_priv", f"private-{sums}",
+                {"private_accumulators": rp["accumulators"], "threads": rp["threads"], "ring_bytes": rp["ring_bytes"]})
+    ring = {"chunk_entries": st["chunk_entries"], "chunk_rows": st["chunk_rows"], "stages": st["stages"],
+            "threads": rp["threads"]}
+    if st["row_path"] == 4:
+        wide = "" if st["ring_threads"] in (0, 1024) else f"-{st['ring_threads']}t"
+        return "k_rowpass_tma", f"bundled-{sums}{wide}", ring
+    return {1: ("k_rowpass", "register", ring), 2: ("k_rowpass_tma", "ring", ring),
+            3: ("k_rowpass_stream", "stream", ring)}[st["row_path"]]
+
+
 def dvh_report(doses, labels, levels=None, names=STRUCTURE_NAMES):
     """DVH bands and dose metrics over the scenarios (the report of Sec. 3.2,
     on synthetic structures).  doses: [N, m] physical dose per scenario (Gy),
@@ -566,9 +582,7 @@ def main():
     # DRAM bytes of one launch from a stored ncu capture of this kernel on this
     # workload (dram__bytes_read.sum + dram__bytes_write.sum), keyed by the kernel
     # variant; null when no capture of the variant in use is stored
-    variant = ("bundled-" + ("exact" if st["exact_sums"] else "float") +
-               ("" if st["ring_threads"] in (0, 1024) else f"-{st['ring_threads']}t") if st["row_path"] == 4
-               else {1: "register", 2: "ring", 3: "stream"}[st["row_path"]])
+    kernel, variant, pass_cfg = row_pass_report(st, plan.row_pass())
     traffic, traffic_src = None, None
     tr_path = os.path.join(ROOT, "profiles", "traffic.json")
     if os.path.exists(tr_path):
@@ -589,9 +603,7 @@ def main():
                    "eps_abs": params.eps_abs, "eps_rel": params.eps_rel,
                    "rho": infos[-1]["rho"], "l2": "inputs 1.02 GB > 129 MB L2, no flush",
                    "parallelism": "replicas" if world > 1 else "single GPU", "seed": args.seed,
-                   "ring": {"chunk_entries": st["chunk_entries"], "chunk_rows": st["chunk_rows"],
-                            "stages": st["stages"], "threads": st["ring_threads"],
-                            "configs_timed": st["autotuned"]}},
+                   "row_pass": {**pass_cfg, "configs_timed": st["autotuned"]}},
         "admm": {"f_rel_gap_vs_exact": (None if _golden_fstar() is None or args.seed != 0
                                         else (infos[-1]["f"] - _golden_fstar()) / _golden_fstar()),
                  "iterations": iters, "cg_iterations": statistics.mean(i["inner"] for i in infos),
@@ -601,9 +613,7 @@ def main():
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "traffic_source": traffic_src or "no stored capture of this kernel variant",
-                     "kernel": ({4: "k_rowpass_priv (k_rowpass_tma where its accumulators don't fit)",
-                                 2: "k_rowpass_tma"}.get(st["row_path"], "k_rowpass")) +
-                               f"<kNormal,f32,int32,{variant}> (CG operator pass, all scenarios)",
+                     "kernel": f"{kernel}<kNormal,f32,int32,{variant}> (CG operator pass, all scenarios)",
                      "ms_per_launch": ms_pass, "bytes_per_launch": bytes_pass,
                      "bytes_note": ("bundled layout: stored block columns (4 values + 1 index, 20 B) and 64-byte "
                                     "bundle records, plus the spot vectors in and out"
@@ -666,8 +676,8 @@ def main():
             fe1.record(stream)
             torch.cuda.synchronize(dev)
             f_on_f32 = plan.objective(zf)
-            sf = pf.stats()
-            forms[name] = {"ring": [sf["chunk_entries"], sf["stages"], sf["ring_threads"]],
+            kf, vf_, cf = row_pass_report(pf.stats(), pf.row_pass())
+            forms[name] = {"row_pass": {"kernel": f"{kf}<{vf_}>", **cf},
                            "ms_per_pass": ms_f, "bytes_per_pass": by_f, "gbs": by_f / ms_f / 1e6,
                            "frac_of_peak": by_f / ms_f / 1e6 / peak,
                            "solve_s": fe0.elapsed_time(fe1) / 1e3, "iterations": fi["iterations"],
@@ -788,9 +798,10 @@ def main():
                       "iterations": e2e_it,
                       "phases_s": {k: statistics.mean(p[i] for p in phases) for i, k in
                                    enumerate(("create_host_layout", "create_device", "create_autotune", "solve"))},
-                      "note": "plan_create from host CSR (validate, bundle, upload, autotune the ring) + solve + "
-                              "x read-back; mean over runs (the iteration count of a solve varies by a few "
-                              "percent with the order of floating-point atomics)"}
+                      "note": "plan_create from host CSR (validate, bundle, upload, autotune the row pass) + solve + "
+                              "x read-back; mean over runs (private accumulators add in a fixed order, so solves "
+                              "take the same iterations; where the ring is in use, the order of its atomics "
+                              "varies them by a few percent)"}
 
     if rank == 0 and world == 1 and not args.no_cpu:
         out["cpu_baseline"] = cpu_baseline(prob, budget_s=args.cpu_budget)

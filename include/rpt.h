@@ -204,8 +204,8 @@ typedef struct {
   int32_t sm_count;
   double  default_rho;    /* 2 mean_s(trace(A~_s^T A~_s))/n (without rho_scale) */
   double  const_term;     /* sum over rows not stored for a scenario of c_s w_i p_i^2 (part of every f) */
-  int32_t row_path;       /* row-pass implementation in use: 1 register-direct, 2 bulk-copy ring, 3 streaming,
-                             4 bundled ring */
+  int32_t row_path;       /* row-pass layout in use: 1 register-direct, 2 bulk-copy ring, 3 streaming,
+                             4 bundled rows (by which pass: rpt_plan_row_pass_query) */
   int32_t min_lanes;      /* smallest lanes-per-row group */
   int32_t chunk_entries;  /* ring / streaming: entries per chunk (0 for the register path) */
   int32_t chunk_rows;     /* ring / streaming: rows per chunk */
@@ -218,7 +218,7 @@ typedef struct {
                              are entries of the matrix */
   int32_t exact_sums;     /* 1: the row passes sum in exact fixed point (path 4 with accumulate 1), so
                              their results do not depend on scheduling; 0: float atomics */
-  int32_t ring_threads;   /* path 4: threads of a row-pass CTA (1024, 768 or 640); 0 otherwise */
+  int32_t ring_threads;   /* path 4: threads of a CTA of the ring (1024, 768 or 640); 0 otherwise */
   /* wall time of rpt_plan_create by phase (seconds): */
   double  layout_seconds;   /* host: validation, row compaction and the stored layout */
   double  device_seconds;   /* device set-up, allocation, upload and device-side preparation */
@@ -260,7 +260,16 @@ int rpt_plan_set_weights(rpt_plan* plan, const double* voxel_w, const double* pr
 /* Release a plan and its device memory.  NULL is accepted. */
 void rpt_plan_destroy(rpt_plan* plan);
 
+/* The fields row_path .. ring_threads of rpt_plan_stats describe the stored layout
+ * and, for path 4, the ring (which the modes of a plan without private
+ * accumulators use); rpt_plan_row_pass_query says which pass runs. */
 int rpt_plan_query(const rpt_plan* plan, rpt_plan_stats* out);
+
+/* The row pass in use (all pointers may be NULL): *accumulators: private
+ * accumulators of a CTA (row path 4; 0: the pass of row_path with atomics);
+ * *threads: threads of a CTA; *ring_bytes: bytes of its ring beside the private
+ * accumulators (0 without them). */
+int rpt_plan_row_pass_query(const rpt_plan* plan, int32_t* accumulators, int32_t* threads, int32_t* ring_bytes);
 
 /* ---- batched plans: several problems in one plan and one launch per pass ----
  *

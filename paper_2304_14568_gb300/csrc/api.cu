@@ -1443,6 +1443,19 @@ int rpt_plan_query(const rpt_plan* plan, rpt_plan_stats* out) {
   return RPT_OK;
 }
 
+int rpt_plan_row_pass_query(const rpt_plan* plan, int32_t* accumulators, int32_t* threads, int32_t* ring_bytes) {
+  if (!plan) {
+    set_error("null argument");
+    return RPT_EINVAL;
+  }
+  const DevPlan& dp = reinterpret_cast<const Plan*>(plan)->dp;
+  const bool priv = use_priv(dp);
+  if (accumulators) *accumulators = priv ? dp.priv_acc : 0;
+  if (threads) *threads = rowpass_threads(dp);
+  if (ring_bytes) *ring_bytes = priv ? dp.ring_bytes : 0;
+  return RPT_OK;
+}
+
 int rpt_admm_bb_solve(rpt_plan* plan, const rpt_admm_params* params, const double* z0,
                       const double* y0, double* x_out, rpt_solve_info* info) {
   if (!plan || !params) {

@@ -29,7 +29,7 @@ EXPORTED = [
     "rpt_mlp_get_params", "rpt_mlp_set_params", "rpt_mlp_loss_grad", "rpt_mlp_train", "rpt_mlp_predict",
     "rpt_admm_bb_solve_learned", "rpt_trace_get", "rpt_plans_create_batched", "rpt_plan_batch_query",
     "rpt_admm_bb_solve_batched", "rpt_mlp_infer", "rpt_mlp_set_compute", "rpt_plan_set_weights",
-    "rpt_admm_bb_solve_constrained",
+    "rpt_admm_bb_solve_constrained", "rpt_plan_row_pass_query",
 ]
 
 
@@ -138,6 +138,8 @@ def lib():
     L.rpt_plan_destroy.restype = None
     L.rpt_plan_query.argtypes = [C.c_void_p, C.POINTER(_Stats)]
     L.rpt_plan_query.restype = C.c_int
+    L.rpt_plan_row_pass_query.argtypes = [C.c_void_p] + [C.POINTER(C.c_int32)] * 3
+    L.rpt_plan_row_pass_query.restype = C.c_int
     L.rpt_admm_bb_solve.argtypes = [C.c_void_p, C.POINTER(AdmmParams), dp, dp, dp, C.POINTER(_Info)]
     L.rpt_admm_bb_solve.restype = C.c_int
     L.rpt_pgd_solve.argtypes = [C.c_void_p, C.POINTER(PgdParams), dp, dp, C.POINTER(_Info)]
@@ -380,6 +382,13 @@ class Plan:
         s = _Stats()
         _check(lib().rpt_plan_query(self._h, C.byref(s)))
         return s.as_dict()
+
+    def row_pass(self) -> dict:
+        """The row pass in use (rpt_plan_row_pass_query): private accumulators of a CTA
+        (0: the pass with atomics), its threads, the bytes of the ring beside them."""
+        v = [C.c_int32() for _ in range(3)]
+        _check(lib().rpt_plan_row_pass_query(self._h, *[C.byref(a) for a in v]))
+        return dict(zip(("accumulators", "threads", "ring_bytes"), (a.value for a in v)))
 
     def admm_bb_solve(self, params: AdmmParams | None = None, z0=None, y0=None, **kw):
         prm = params if params is not None else admm_params(**kw)
