@@ -67,8 +67,9 @@ struct DevPlan {
   const int4* blocks;                 // path 0: [grid] (s, first row, end row, lanes per row)
   // Partial slots of the last pass, per scenario: slot_count[s] slots listed in
   // slot_list[s * slot_cap ...] in increasing order (static for path 0, written
-  // by the finishing CTA of every pass for path 1); objs[s] = objective of
-  // scenario s in the last objective pass.
+  // by the finishing CTA of every pass with a queue); the pass with private
+  // accumulators lists the first only, as its slots are consecutive.  objs[s] =
+  // objective of scenario s in the last objective pass.
   int* slot_count;                    // [N]
   int* slot_list;                     // [N][slot_cap]
   double* objs;                       // [N]

@@ -14,8 +14,8 @@
 //   op(A)(i,k) = TA ? A[k*lda + i] : A[i*lda + k];  op(B)(k,j) = TB ? B[j*ldb + k] : B[k*ldb + j]
 // with the structure flags of gemm.cuh:
 //   lower: compute only output tiles that reach the lower triangle (j <= i);
-//   kdiag 1: op(B)(k, j) is zero for k < j (K starts at the tile's first column);
-//   kdiag 2: also op(A)(i, k) is zero for k < i (K starts at max of both);
+//   kdiag 2: op(B)(k, j) is zero for k < j and op(A)(i, k) for k < i (K starts at the
+//     later of the tile's first column and row);
 //   kdiag 3: op(A)(i, k) is zero for k < i (K starts at the tile's first row);
 //   kdiag 4: op(A)(i, k) is zero for k > i (K ends with the tile's last row).
 // Several products per batch entry (T3Pairs): product p of an entry works p steps
@@ -98,7 +98,7 @@ k_gemm_tf32x3(int M, int N, int K, const float* A, int lda, long long sA, const 
     for (int b = 0; b < 4; ++b)
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-  const int kfirst = kdiag == 2 ? max(i0, j0) : (kdiag == 1 ? j0 : (kdiag == 3 ? i0 : 0));
+  const int kfirst = kdiag == 2 ? max(i0, j0) : (kdiag == 3 ? i0 : 0);
   constexpr int kPer = kT3BM * kT3BK / kT3Threads;   // tile elements per thread and operand (16)
   float ra[kPer], rb[kPer];
   // loads run along each operand's contiguous dimension

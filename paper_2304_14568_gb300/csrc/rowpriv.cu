@@ -343,7 +343,7 @@ k_rowpass_priv(DevPlan P, const float* __restrict__ vin, int v_stride, const int
         if (u > 0) {
           const int b0 = (int)(((long long)(pre + 1) * G - 1) / T), b1 = (int)(((long long)(pre + u) * G - 1) / T);
           cnt = b1 - b0 + 1;
-          for (int k = 0; k < cnt; ++k) P.slot_list[(size_t)s * P.slot_cap + k] = b0 + rank + k;
+          P.slot_list[(size_t)s * P.slot_cap] = b0 + rank;   // the first; the others follow it
         }
         P.slot_count[s] = cnt;
       }
