@@ -115,6 +115,7 @@ k_noalloc_pass(int m, int n, int n_pad, int apart, const int32_t* __restrict__ r
       blo = __ldg(rp + i);
       bhi = __ldg(rp + i + 1);
       if (bhi > blo) bw = __ldg(w + i);
+      else bhi = blo;        // (offsets that decrease: an empty row; the entries are counted unsigned)
     }
     const unsigned any = __ballot_sync(0xffffffffu, bhi > blo);
     for (int b = 0; b < kNaBatch; ++b) {
