@@ -371,7 +371,7 @@ k_rowpass_tma(DevPlan P, const float* __restrict__ vin, int v_stride, const int*
       }
     };
     for (;;) {
-      if (!mbar_wait(smem_u32(&full[st]), (uint32_t)ph)) {
+      if (!warp_mbar_wait(smem_u32(&full[st]), (uint32_t)ph)) {
         if (lane == 0) atomicExch(P.err, 3);
         break;
       }

@@ -19,10 +19,10 @@ def _raw_waits(src):
     return [m.start() for m in re.finditer(r"(?<![\w])(mbar_wait|flag_wait)\(", src)], src
 
 
-@pytest.mark.parametrize("name", ["rowpriv.cu"])
+@pytest.mark.parametrize("name", ["rowpriv.cu", "rowpass.cu"])
 def test_consumers_take_one_answer_a_warp(name):
     at, src = _raw_waits(_source(name))
-    consumers = src.index("int cw = warp - ")
+    consumers = src.index("int cw = warp - ")       # producers come before
     assert not [a for a in at if a > consumers], name
 
 
