@@ -92,9 +92,9 @@ typedef struct {
                                          spot index per column of a group (rows that are neighbours in the
                                          input order should share spots, as voxels in grid order do); see
                                          accumulate for its exact (bitwise reproducible) sums.  The pass
-                                         adds into private accumulators where they fit (plans of one problem
-                                         that set no ring geometry or ring_threads), else with atomics
-                                         behind a ring;
+                                         adds into private accumulators where they fit and are the faster way
+                                         (plans of one problem that set no ring geometry or ring_threads;
+                                         rpt_plan_row_pass_query tells), else with atomics behind a ring;
                                        0: 4 when its shared-memory stage fits the plan, else 2, else 1 */
   int32_t autotune;                 /* 1: time every ring configuration that fits this plan (entries and
                                        rows per stage, stages) on its own row pass and keep the fastest;

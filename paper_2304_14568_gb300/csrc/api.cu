@@ -185,10 +185,10 @@ using namespace layout;   // lanes per row, row lists, bank balance, chunks (lay
 // Pass with private accumulators: consumer warps, bytes that its ring has at
 // least, units cut per CTA.  Twelve warps beat ten (0.166 against 0.187 ms on the
 // realistic plan) and leave 128 registers a thread.  Fewer accumulators make room
-// for the ring but more warps wait for a turn: with a ring of 72 KB (six
-// accumulators) the realistic plan took 0.213 ms against 0.166 with 128 KB (four);
-// twelve against six accumulators cost 0.066 against 0.057 ms at 2000 spots, three
-// against two gain 0.066 against 0.071 at 7000.
+// for the ring but more warps wait for a turn: the realistic plan takes 0.193 ms with six
+// and 84 KB of ring, 0.153 with four and 123 KB, 0.168 with three and 143 KB, 0.256 with
+// two and 163 KB; 2000 spots 0.057 with six (166 KB), 0.070 with three, 0.100 with two; 7000
+// spots 0.072 with four (84 KB), 0.066 with three (112 KB), 0.091 with two.
 constexpr int kPrivWarps = 12;
 constexpr size_t kPrivRing = 98304;
 constexpr int kUnitsPerCta = 64;
@@ -762,12 +762,13 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
     dp.grid = P->sm_count * ctas;
     dp.nblocks = dp.grid * N;
     dp.slot_cap = dp.grid;
-    // private accumulators, unless the caller set the ring's geometry; at least two
-    // beside a ring of kPrivRing bytes (about 10,500 spots), three with fixed-point
-    // sums (4,600 spots), which hold their turn longer: at 5000 spots two took 0.294
-    // ms against the ring's 0.267.  Batched plans keep the ring: with three CTAs or so
-    // to a unit the float sums are grouped so differently that the iterates of a
-    // batched solve move by more than the ring's spread from run to run.
+    // private accumulators, unless the caller set the ring's geometry: the most that fit
+    // beside a ring of kPrivRing bytes (two up to about 10,500 spots; with fixed-point sums
+    // three up to 4,500, as two, which hold their turn longer, lost to the ring: 0.294 against
+    // 0.267 ms at 5000 spots), where they beat the ring by private_sums_pay or, when
+    // autotuning, by the clock.  Batched plans keep the ring: their passes with private
+    // accumulators took two thirds of the time and came nearer to the exact sums, but moved
+    // the iterates of a batched solve by 1 to 4e-6, more than two runs of the ring differ by.
     if (G == 1 && !want_thr && ring_override(opts, 1, 1, 2).empty()) {
       int widest = 0;
       cut_units(R, N, (int64_t)dp.grid * kUnitsPerCta, 4 * bv + bi, &icls, &ubeg, &uoff, &widest);
@@ -778,6 +779,9 @@ int create_plan(const rpt_problem* pr, const rpt_device_opts* opts, rpt_plan** o
       for (int a : {6, 4, 3, 2}) {     // accumulators of the 12 consumer warps
         const size_t fixed = priv_fixed_bytes(n_pad, a, exact);
         if (fixed + std::max(kPrivRing, 2 * item) > room || (exact && a < 3)) continue;
+        if (!autotune && !private_sums_pay(a, exact, pr->value_format, NE / dp.grid,
+                                           NE / std::max<int64_t>(1, n_bundles), dp.cmax))
+          break;
         dp.priv = kPrivWarps;
         dp.priv_acc = a;
         dp.ring_bytes = (int)std::min((room - fixed) & ~(size_t)127, (size_t)1 << 18);

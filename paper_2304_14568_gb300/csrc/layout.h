@@ -508,5 +508,27 @@ inline void cut_units(const RowLists& R, int N, int64_t parts, int col_bytes, st
   (*uoff)[N] = (int)ubeg->size();
 }
 
+// Whether the pass with `accs` private accumulators is the better one, against the ring
+// whose stage holds ring_cols block columns; cols_per_cta, width: block columns a CTA
+// and a bundle on average.  Few accumulators make the warps wait for turns, so
+//  * float sums with three or more always win (1.05 to 2.6 times, 200 to 8000 spots);
+//  * with two (8,100 to 10,500 spots) they win on little work a CTA (38.4 us against 41.6 at
+//    39,000 columns a CTA in BF16, 20.5 against 26 at 12,000), on wide bundles, whose ends the ring
+//    reads twice (F32 and FP8 from 300 block columns on: 110.5 against 113.9 and 94.9 against
+//    95.9 us at 312, 93 against 112 and 76 against 90 at 428; BF16 from 400 on: 98 against 91 at
+//    312, 83 against 90 at 428), and where the ring's stages are cut short (F32 beyond 9,900
+//    spots: 256 against 429); on narrow bundles they lose (9000 spots, 195 a bundle: F32 245
+//    against 210, BF16 219 against 170, FP8 208 against 179);
+//  * exact sums with three or four are even or better in F32 and BF16 (0.95 to 1.18 times);
+//    FP8 values add so fast that turns of 64-bit sums are all they wait for: 123 us
+//    against 111 (4400 spots), 159 against 152 (3000), but 27 against 39 at 18,000 columns a CTA.
+inline bool private_sums_pay(int accs, bool exact, int value_format, int64_t cols_per_cta, int64_t width,
+                             int ring_cols) {
+  constexpr int kBf16 = 1, kFp8 = 2;
+  if (exact) return value_format != kFp8 || accs >= 6 || cols_per_cta <= 20000;
+  if (accs >= 3 || cols_per_cta <= 40000 || ring_cols < 3072) return true;
+  return width >= (value_format == kBf16 ? 400 : 300);
+}
+
 }  // namespace layout
 }  // namespace rpt

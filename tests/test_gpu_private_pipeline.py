@@ -40,9 +40,15 @@ def _short(n, seed):
 
 def _wide(n, seed):
     """15,000 bundles of 32 lanes, a quarter of them past 384 columns: 100 items a CTA, 0.8 MB
-    through a ring of 100 to 130 KB (half as much and less in the quantised forms)."""
+    through a ring of 100 to 130 KB (half as much in BF16)."""
     rng = np.random.default_rng(seed)
     return _matrix(np.concatenate([rng.integers(97, 385, size=11_000), rng.integers(385, 800, size=4_000)]), n, seed)
+
+
+def _wide_fp8(n, seed):
+    """As many as exact FP8 sums take with fewer than six accumulators (20,000 columns a CTA)."""
+    rng = np.random.default_rng(seed)
+    return _matrix(np.concatenate([rng.integers(97, 385, size=6_000), rng.integers(385, 800, size=2_200)]), n, seed)
 
 
 def _plan(rpt, mats, n, **kw):
@@ -57,13 +63,14 @@ def _plan(rpt, mats, n, **kw):
 def matrices():
     # spots, accumulators of exact sums, matrices (two scenarios of the short bundles)
     return {"short": (250, 6, [_short(250, 1), _short(250, 2)]), "wide4": (3400, 4, [_wide(3400, 3)]),
-            "wide3": (4500, 3, [_wide(4500, 4)])}
+            "wide3": (4500, 3, [_wide(4500, 4)]), "wide4_fp8": (3400, 4, [_wide_fp8(3400, 3)]),
+            "wide3_fp8": (4500, 3, [_wide_fp8(4500, 4)])}
 
 
 @pytest.mark.parametrize("case", ["short", "wide4", "wide3"])
 @pytest.mark.parametrize("fmt,iw", [(0, 32), (0, 16), (1, 32), (1, 16), (2, 32), (2, 16)])
 def test_exact_sums_have_the_rings_bits(rpt, matrices, case, fmt, iw):
-    n, accs, mats = matrices[case]
+    n, accs, mats = matrices[case + ("_fp8" if fmt == 2 and case != "short" else "")]
     N = len(mats)
     rng = np.random.default_rng(5)
     V = rng.normal(size=(N, n))
@@ -81,6 +88,24 @@ def test_exact_sums_have_the_rings_bits(rpt, matrices, case, fmt, iw):
         assert np.array_equal(a, b)
     assert np.array_equal(got[0][0], got[0][3])
     np.testing.assert_allclose(fs[0], fs[1], rtol=1e-12)
+
+
+@pytest.mark.parametrize("fmt,exact,n,accs", [(0, 0, 9000, 0), (1, 0, 9000, 0), (2, 0, 9000, 0), (2, 1, 3400, 0),
+                                              (0, 1, 3400, 4), (1, 0, 7000, 3)])
+def test_narrow_bundles_keep_the_ring_where_it_is_faster(rpt, fmt, exact, n, accs):
+    """8 M block columns of 100 a bundle on average: two accumulators, and FP8's exact sums
+    with fewer than six, would wait for turns longer than the ring's atomics take."""
+    rp, ci, va = _matrix(np.random.default_rng(1).integers(60, 141, size=82_000), n, 8)
+    P, w = _plan(rpt, [(rp, ci, va)], n, accumulate=1 if exact else 2, value_format=fmt, index_width=16)
+    with P:
+        assert P.stats()["block_cols"] / 152 > 40_000
+        assert P.row_pass()["accumulators"] == accs
+        V = np.random.default_rng(6).normal(size=n)
+        U = np.asarray(P.apply_normal(V, 0.7)).reshape(-1)
+    if fmt == 0:
+        A = sp.csr_matrix((va.astype(np.float64), ci, rp), shape=(len(rp) - 1, n))
+        ref = A.T @ (w * (A @ V)) + 0.35 * V
+        assert np.linalg.norm(U - ref) <= 1e-5 * np.linalg.norm(ref)
 
 
 @pytest.mark.parametrize("n,accs,make", [(250, 6, _short), (4500, 6, _wide), (5000, 4, _wide), (7000, 3, _wide),
