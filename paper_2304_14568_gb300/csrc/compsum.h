@@ -18,6 +18,10 @@ struct CompSum {
     c += (s - (t - b)) + (p - b);
     s = t;
   }
+  RPT_HD void add(const CompSum& o) {
+    add(o.s);
+    c += o.c;
+  }
   RPT_HD double value() const { return (double)s + (double)c; }
 };
 

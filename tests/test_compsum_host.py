@@ -25,6 +25,8 @@ def shim(tmp_path_factory):
     L = C.CDLL(out)
     L.shim_compsum.restype = C.c_double
     L.shim_compsum.argtypes = [np.ctypeslib.ndpointer(np.float32, flags="C"), C.c_int]
+    L.shim_compsum_parts.restype = C.c_double
+    L.shim_compsum_parts.argtypes = [np.ctypeslib.ndpointer(np.float32, flags="C"), C.c_int, C.c_int]
     return L
 
 
@@ -44,9 +46,20 @@ def test_as_good_as_a_float64_sum(shim, n, spread):
         assert worst < 2.0 ** -36 < worst32
 
 
+@pytest.mark.parametrize("n", [1, 40, 157, 1000])
+@pytest.mark.parametrize("parts", [2, 32, 64])
+def test_sums_added_up_are_as_good(shim, n, parts):
+    rng = np.random.default_rng(n)
+    for _ in range(20):
+        p = rng.normal(size=n).astype(np.float32)
+        exact, mag = float(np.sum(p.astype(np.longdouble))), float(np.sum(np.abs(p).astype(np.float64)))
+        assert abs(shim.shim_compsum_parts(p, n, parts) - exact) <= (2.0 ** -50 + (n * 2.0 ** -24) ** 2) * mag
+
+
 def test_the_x_update_sums_every_product_this_way():
     src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "solver.cu")).read())
     at = src.index("k_chol_x(DevPlan P")
     body = src[at:src.index("__global__", at)]
     assert "CompSum" in body and "__fmul_rn(" in body
     assert not re.search(r"\w\.x \* \w+\.x", body)      # no product enters a plain float32 sum
+    assert "double" not in body.split("CompSum sum[4]")[1]  # and a row needs no float64 sum (two lanes a cycle)
