@@ -38,11 +38,14 @@ constexpr int kNaLanes = 8;                // lanes per row
 constexpr int kNaKeep = 16;                // entries per lane kept between the dot and the scatter
 constexpr int kNaApart = 1024;             // the 4 rows of a warp step lie up to this far apart
 constexpr int kNaBatch = 8;                // steps whose row offsets are loaded together
+constexpr int kNaTail = 8;                 // entries of a longer row, per lane, loaded together (few rows)
+constexpr int kNaFew = 8192;               // up to so many rows each is a step of its own, for a whole warp
 
 // One row by L lanes (this lane is sl), or nothing when lo == hi: the row's
 // entries, the first KEEP L of them kept in registers between the dot and the
-// scatter.  Entries outside [0, n) are ignored.  Every lane of the warp calls it.
-template <int L, int KEEP>
+// scatter, and TAIL of the further ones loaded at a time.  Entries outside [0, n) are
+// ignored.  Every lane of the warp calls it.
+template <int L, int KEEP, int TAIL>
 __device__ __forceinline__ void na_row(unsigned lo, unsigned hi, unsigned sl, float wi, int n, const int32_t* __restrict__ col,
                                        const float* __restrict__ val, const float* sv, float* acc) {
   float a[KEEP];
@@ -57,9 +60,24 @@ __device__ __forceinline__ void na_row(unsigned lo, unsigned hi, unsigned sl, fl
 #pragma unroll
   for (int k = 0; k < KEEP; ++k)
     if ((unsigned)c[k] < (unsigned)n) t = fmaf(a[k], sv[c[k]], t);
-  for (unsigned e = lo + sl + L * KEEP; e < hi; e += L) {
-    const int q = __ldg(col + e);
-    if ((unsigned)q < (unsigned)n) t = fmaf(__ldg(val + e), sv[q], t);
+  if constexpr (TAIL == 1) {
+    for (unsigned e = lo + sl + L * KEEP; e < hi; e += L) {
+      const int q = __ldg(col + e);
+      if ((unsigned)q < (unsigned)n) t = fmaf(__ldg(val + e), sv[q], t);
+    }
+  } else {
+    for (unsigned e = lo + sl + L * KEEP; e < hi; e += L * TAIL) {
+      float b[TAIL];
+      int q[TAIL];
+#pragma unroll
+      for (int k = 0; k < TAIL; ++k) {
+        b[k] = e + L * k < hi ? __ldg(val + e + L * k) : 0.f;
+        q[k] = e + L * k < hi ? __ldg(col + e + L * k) : -1;
+      }
+#pragma unroll
+      for (int k = 0; k < TAIL; ++k)
+        if ((unsigned)q[k] < (unsigned)n) t = fmaf(b[k], sv[q[k]], t);
+    }
   }
 #pragma unroll
   for (int o = L / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -67,9 +85,24 @@ __device__ __forceinline__ void na_row(unsigned lo, unsigned hi, unsigned sl, fl
 #pragma unroll
   for (int k = 0; k < KEEP; ++k)
     if ((unsigned)c[k] < (unsigned)n) atomicAdd(&acc[c[k]], coef * a[k]);
-  for (unsigned e = lo + sl + L * KEEP; e < hi; e += L) {
-    const int q = __ldg(col + e);
-    if ((unsigned)q < (unsigned)n) atomicAdd(&acc[q], coef * __ldg(val + e));
+  if constexpr (TAIL == 1) {
+    for (unsigned e = lo + sl + L * KEEP; e < hi; e += L) {
+      const int q = __ldg(col + e);
+      if ((unsigned)q < (unsigned)n) atomicAdd(&acc[q], coef * __ldg(val + e));
+    }
+  } else {
+    for (unsigned e = lo + sl + L * KEEP; e < hi; e += L * TAIL) {
+      float b[TAIL];
+      int q[TAIL];
+#pragma unroll
+      for (int k = 0; k < TAIL; ++k) {
+        b[k] = e + L * k < hi ? __ldg(val + e + L * k) : 0.f;
+        q[k] = e + L * k < hi ? __ldg(col + e + L * k) : -1;
+      }
+#pragma unroll
+      for (int k = 0; k < TAIL; ++k)
+        if ((unsigned)q[k] < (unsigned)n) atomicAdd(&acc[q[k]], coef * b[k]);
+    }
   }
 }
 
@@ -81,11 +114,18 @@ __device__ __forceinline__ void na_row(unsigned lo, unsigned hi, unsigned sl, fl
 // neighbouring rows share most of their spots, and lanes that meet on one spot
 // retry their atomics.  Row offsets are loaded for kNaBatch steps at once; empty
 // steps cost a ballot.  Rows longer than the 8 lanes keep in registers are left
-// for the whole warp.  One scenario of the realistic plan (10.0 M entries, 299k
+// for the whole warp.  A matrix of few rows (kNaFew) has a step and a warp for each row,
+// on as many CTAs as there are rows: with 4 rows a step, half as many warps and one of
+// them after the other, 100 rows of 8000 entries took 607 us, 1000 of 2000 158 (103 and 56
+// cut by entries), against
+// 33 and 20.5 us; the line lies where short rows would gain by sharing a warp (10,000 rows of 10
+// entries 10.6 us shared, 14.7 apart; 6000 of 200 16.7 and 14.5).  (kNaTail loads at a time
+// in the other form cost its short rows 4 %.)  One scenario of the realistic plan (10.0 M entries, 299k
 // rows of which 214k are empty, 5000 spots): 52 us for both kernels against
 // 2568 us when CTAs were cut by entries, which left the empty rows at both ends
 // of the volume to two CTAs, and each warp waited for one row at a time; 190k
 // entries and 200 spots: 12 us against 49 us.
+template <int ROWS>
 __global__ void __launch_bounds__(kNaThreads)
 k_noalloc_pass(int m, int n, int n_pad, int apart, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
                const float* __restrict__ val, const float* __restrict__ w, const float* __restrict__ v,
@@ -100,18 +140,18 @@ k_noalloc_pass(int m, int n, int n_pad, int apart, const int32_t* __restrict__ r
   }
   __syncthreads();
   const int sl = lane & (kNaLanes - 1);
-  const int tile = 4 * apart;
-  const int steps = ((m - 1) / tile + 1) * apart;   // m / 4 rounded up to whole tiles
+  const int tile = ROWS * apart;
+  const int steps = ((m - 1) / tile + 1) * apart;   // m / ROWS rounded up to whole tiles
   const int stride = gridDim.x * nw;
   // consecutive steps go to different CTAs
   const int first = (tid >> 5) * gridDim.x + blockIdx.x;
   for (int s0 = first; s0 < steps; s0 += stride * kNaBatch) {
-    // lane l: row l & 3 of the batch's step l >> 2
+    // lane l: row l & 3 (of ROWS) of the batch's step l >> 2
     const int s = s0 + stride * (lane >> 2);
     const long long i = (long long)(s / apart) * tile + s % apart + (lane & 3) * apart;
     int blo = 0, bhi = 0;
     float bw = 0.f;
-    if (s < steps && i < m) {
+    if (s < steps && i < m && (lane & 3) < ROWS) {
       blo = __ldg(rp + i);
       bhi = __ldg(rp + i + 1);
       if (bhi > blo) bw = __ldg(w + i);
@@ -123,13 +163,13 @@ k_noalloc_pass(int m, int n, int n_pad, int apart, const int32_t* __restrict__ r
       const int from = 4 * b + lane / kNaLanes;
       const int lo = __shfl_sync(0xffffffffu, blo, from), hi = __shfl_sync(0xffffffffu, bhi, from);
       const float wi = __shfl_sync(0xffffffffu, bw, from);
-      const bool wide = hi - lo > kNaLanes * kNaKeep;
-      na_row<kNaLanes, kNaKeep>(lo, wide ? lo : hi, sl, wi, n, col, val, sv, acc);
+      const bool wide = ROWS == 1 ? hi > lo : hi - lo > kNaLanes * kNaKeep;
+      if (ROWS > 1) na_row<kNaLanes, kNaKeep, 1>(lo, wide ? lo : hi, sl, wi, n, col, val, sv, acc);
       unsigned left = __ballot_sync(0xffffffffu, wide && sl == 0);
       while (left) {
         const int src = __ffs(left) - 1;
         left &= left - 1;
-        na_row<32, kNaKeep>(__shfl_sync(0xffffffffu, lo, src), __shfl_sync(0xffffffffu, hi, src), lane,
+        na_row<32, kNaKeep, ROWS == 1 ? kNaTail : 1>(__shfl_sync(0xffffffffu, lo, src), __shfl_sync(0xffffffffu, hi, src), lane,
                             __shfl_sync(0xffffffffu, wi, src), n, col, val, sv, acc);
       }
     }
@@ -220,18 +260,19 @@ extern "C" int rpt_normal_apply_noalloc(int32_t m, int32_t n, const int32_t* row
   }
   const int n_pad = (n + 31) / 32 * 32;
   const size_t smem = (size_t)n_pad * 2 * sizeof(float);
-  if ((e = cudaFuncSetAttribute(k_noalloc_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+  const bool few = m <= kNaFew;
+  auto* pass = few ? k_noalloc_pass<1> : k_noalloc_pass<4>;
+  if ((e = cudaFuncSetAttribute(pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
     return cuda_fail(e, "kernel attribute");
   int ctas = 0;
   if ((e = cudaDeviceGetAttribute(&ctas, cudaDevAttrMultiProcessorCount, dev)))
     return cuda_fail(e, "device attribute");
-  // one CTA per SM, as many as have a partial row and steps for half of their warps
+  // one CTA per SM, as many as have a partial row and rows, or steps for half of their warps
   ctas = std::min(ctas, na_ctas(n_pad));
-  const int apart = std::min(kNaApart, m / 4 + 1);
-  ctas = std::min(ctas, (m - 1) / (2 * (kNaThreads / 32)) + 1);
+  const int apart = few ? 1 : std::min(kNaApart, m / 4 + 1);
+  ctas = std::min(ctas, few ? m : (m - 1) / (2 * (kNaThreads / 32)) + 1);
   cudaStream_t st = (cudaStream_t)stream;
-  k_noalloc_pass<<<ctas, kNaThreads, smem, st>>>(m, n, n_pad, apart, row_ptr_dev, col_idx_dev, val_dev, row_w_dev, v_dev,
-                                                 scratch);
+  pass<<<ctas, kNaThreads, smem, st>>>(m, n, n_pad, apart, row_ptr_dev, col_idx_dev, val_dev, row_w_dev, v_dev, scratch);
   if ((e = cudaGetLastError())) return cuda_fail(e, "launch");
   k_noalloc_reduce<<<n_pad / 32, 32 * kNaSums, 0, st>>>(n, n_pad, ctas, scratch, v_dev, (float)(0.5 * rho), u_dev);
   if ((e = cudaGetLastError())) return cuda_fail(e, "launch");
