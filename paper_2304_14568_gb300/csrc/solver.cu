@@ -55,45 +55,60 @@ __device__ __forceinline__ Slots slots_of(const DevPlan& P, int s) {
   return S;
 }
 
+// Sixteen slots at a time: all loads of a batch are issued before `add` takes them in slot
+// order; the last batch's loads beyond the last slot read that again and count as zeros
+// (which change nothing), so that no load hangs on a condition.
+template <typename T, typename At, typename Add>
+__device__ __forceinline__ void each_partial(const T* __restrict__ part, int cnt, At at, Add add) {
+  constexpr int kB = 16;
+  int k = 0;
+  for (; k + kB <= cnt; k += kB) {
+    T v[kB];
+#pragma unroll
+    for (int u = 0; u < kB; ++u) v[u] = __ldcg(part + at(k + u));
+#pragma unroll
+    for (int u = 0; u < kB; ++u) add(v[u]);
+  }
+  if (k < cnt) {
+    T v[kB];
+#pragma unroll
+    for (int u = 0; u < kB; ++u) v[u] = __ldcg(part + at(min(k + u, cnt - 1)));
+#pragma unroll
+    for (int u = 0; u < kB; ++u) add(k + u < cnt ? v[u] : T(0));
+  }
+}
+template <typename T, typename Add>
+__device__ __forceinline__ void each_partial(const DevPlan& P, const T* __restrict__ part, int j, const Slots& S,
+                                             Add add) {
+  const size_t np = P.n_pad;
+  if (S.list)
+    each_partial(part, S.cnt, [&](int k) { return (size_t)S.list[k] * np + j; }, add);
+  else
+    each_partial(part, S.cnt, [&](int k) { return (size_t)(S.first + k) * np + j; }, add);
+}
+
 // Compensated sum, in slot order, of scenario s's row-pass partials at column j.
-// Sixteen slots at a time, the last batch filled up with zeros (which change
-// nothing): all loads of a batch are issued before the (order-preserving) sums
-// consume them.
 __device__ __forceinline__ double sum_partials_of(const DevPlan& P, const float* __restrict__ part, int s, int j,
                                                   const Slots& S) {
-  constexpr int kB = 16;
   if (P.acc64) {
     // bundled path: 64-bit fixed-point partials, summed exactly (every partial
     // and every sum stays below 2^62 in magnitude), then scaled by 2^-fexp[s]
     // and by the column scale of quantised values
-    const long long* pl = reinterpret_cast<const long long*>(part);
     const int fe = __ldcg(&P.fexp[s]);
     long long sum = 0;
-    for (int k = 0; k < S.cnt; k += kB) {
-      long long v[kB];
-#pragma unroll
-      for (int u = 0; u < kB; ++u) v[u] = k + u < S.cnt ? __ldcg(pl + S.at(k + u) * P.n_pad + j) : 0ll;
-#pragma unroll
-      for (int u = 0; u < kB; ++u) sum += v[u];
-    }
+    each_partial(P, reinterpret_cast<const long long*>(part), j, S, [&](long long v) { sum += v; });
     if (fe == kFexpNaN) return __longlong_as_double(0x7ff8000000000000ll);
     double r = ldexp((double)sum, -fe);
     if (P.colscale) r *= (double)P.colscale[(size_t)s * P.n_pad + j];
     return r;
   }
   float sum = 0.f, c = 0.f;
-  for (int k = 0; k < S.cnt; k += kB) {
-    float v[kB];
-#pragma unroll
-    for (int u = 0; u < kB; ++u) v[u] = k + u < S.cnt ? __ldcg(part + S.at(k + u) * P.n_pad + j) : 0.f;
-#pragma unroll
-    for (int u = 0; u < kB; ++u) {
-      float t, e;
-      two_sum(sum, v[u], t, e);
-      sum = t;
-      c += e;
-    }
-  }
+  each_partial(P, part, j, S, [&](float v) {
+    float t, e;
+    two_sum(sum, v, t, e);
+    sum = t;
+    c += e;
+  });
   return (double)sum + (double)c;
 }
 
