@@ -797,25 +797,26 @@ __global__ void k_pgd_init(DevPlan P, const double* __restrict__ x0, int has_x0,
 }
 
 // Sum over all scenarios of the row-pass partials, for 32 columns per block of 32 x
-// kAllRows threads: latency-bound, so thread row y takes scenarios y, y + kAllRows,
-// ... (kAllRows at a time, into shared memory) and row 0 adds each batch in
-// scenario order.  True in the threads that hold a column's sum.  1777 spots, 7
+// all_rows(N) threads: latency-bound, so thread row y takes scenarios y, y + rows,
+// ... (as many at a time as there are rows, into shared memory) and row 0 adds each batch
+// in scenario order.  True in the threads that hold a column's sum.  1777 spots, 7
 // scenarios: 5 us against 38 us for one thread per column.
 constexpr int kAllRows = 16;
+inline int all_rows(int N) { return std::min(N, kAllRows); }
 __device__ __forceinline__ bool sum_all_scenarios(const DevPlan& P, const float* __restrict__ part, int& j,
                                                   double& sum) {
   __shared__ double sh[kAllRows][33];
-  const int c = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int c = threadIdx.x & 31, y = threadIdx.x >> 5, rows = blockDim.x >> 5;
   j = blockIdx.x * 32 + c;
   sum = 0.0;
-  for (int s0 = 0; s0 < P.N; s0 += kAllRows) {
+  for (int s0 = 0; s0 < P.N; s0 += rows) {
     const int s = s0 + y;
     const double v = (s < P.N && j < P.n) ? sum_partials(P, part, s, j) : 0.0;
     __syncthreads();
     sh[y][c] = v;
     __syncthreads();
     if (y == 0)
-      for (int k = 0; k < kAllRows && s0 + k < P.N; ++k) sum += sh[k][c];
+      for (int k = 0; k < rows && s0 + k < P.N; ++k) sum += sh[k][c];
   }
   return y == 0 && j < P.n;
 }
@@ -1293,7 +1294,7 @@ cudaError_t build_admm_graph(Plan* P, int use_obj, int steps) {
 void pgd_head(Exec& e, Plan* P, unsigned long long htrial, int uc) {
   const DevPlan& dp = P->dp;
   rowpass(e, P, kResid, P->vz32, 0, nullptr);
-  launch(e, k_pgd_grad, dim3((dp.n + 31) / 32), dim3(32 * kAllRows), 0, dp, P->ctl, (const float*)P->partial,
+  launch(e, k_pgd_grad, dim3((dp.n + 31) / 32), dim3(32 * all_rows(dp.N)), 0, dp, P->ctl, (const float*)P->partial,
          P->g, htrial, uc);
 }
 
@@ -1822,7 +1823,7 @@ int op_gradient(Plan* P, const double* x, double* g_out, double* f_out) {
   ex.st = P->stream;
   op_stage(ex, P, 1, P->vz32);
   rowpass(ex, P, kResid, P->vz32, 0, nullptr);
-  launch(ex, k_reduce_all, dim3((dp.n + 31) / 32), dim3(32 * kAllRows), 0, dp, (const float*)P->partial, 2.0,
+  launch(ex, k_reduce_all, dim3((dp.n + 31) / 32), dim3(32 * all_rows(dp.N)), 0, dp, (const float*)P->partial, 2.0,
          P->op_host, (const int*)P->err, P->op_host_report);
   if (int rc = op_wait(ex, P, "launch")) return rc;
   std::memcpy(g_out, P->op_host, sizeof(double) * (size_t)dp.n);
@@ -1996,7 +1997,7 @@ int compute_lipschitz(Plan* P, double* L) {
     ex.st = P->stream;
     op_stage(ex, P, 1, P->vz32);
     rowpass(ex, P, kNormal, P->vz32, 0, nullptr);
-    launch(ex, k_reduce_all, dim3((dp.n + 31) / 32), dim3(32 * kAllRows), 0, dp, (const float*)P->partial, 1.0,
+    launch(ex, k_reduce_all, dim3((dp.n + 31) / 32), dim3(32 * all_rows(dp.N)), 0, dp, (const float*)P->partial, 1.0,
            P->op_host, (const int*)P->err, P->op_host_report);
     const cudaError_t e = cudaStreamSynchronize(P->stream);
     if (ex.err) return cuda_fail(ex.err, "launch");
