@@ -493,18 +493,16 @@ __global__ void k_admm_z(DevPlan P, Ctl* C, const double* __restrict__ x, const 
     double acc = 0.0;
     const int end = (gi + 1) * P.Ns;
     for (int s = gi * P.Ns; s < end; s += 8) {   // the loads of eight scenarios in flight, added in order
-      double a[8];
+      double xs[8], ys[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        a[k] = 0.0;
-        if (s + k < end) {
-          const size_t o = (size_t)(s + k) * P.n + j;
-          a[k] = std_form ? fma(y[o], ir, x[o]) : x[o];
-        }
+      for (int k = 0; k < 8; ++k) {               // (those beyond the last read it again: no load hangs on a condition)
+        const size_t o = (size_t)min(s + k, end - 1) * P.n + j;
+        xs[k] = x[o];
+        ys[k] = y[o];
       }
 #pragma unroll
       for (int k = 0; k < 8; ++k)
-        if (s + k < end) acc += a[k];
+        if (s + k < end) acc += std_form ? fma(ys[k], ir, xs[k]) : xs[k];
     }
     if (live) {
       const double zn = clampd(acc / (double)P.Ns, lo, hi);
