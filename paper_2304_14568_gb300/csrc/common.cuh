@@ -24,12 +24,16 @@
 //               partial slot per scenario it visited (slot = cta * N + s).
 //   path 2 (streaming): the same chunk queues (chunks cut by row-length class),
 //               but every warp of the persistent CTA claims chunks on its own.
-//   path 3 (bundled ring): the ring of path 1 over row bundles (layout.h):
-//               rows grouped 4 at a time, one spot index per block column of a
-//               bundle, records of 4 int4 per bundle; 64-bit fixed-point
-//               accumulators (exact, order-independent sums).
-//   The CTA that finishes last compacts the slots of every scenario into an
-//   ordered list, sums the objective per scenario and resets the queues.
+//   path 3 (row bundles, layout.h): rows grouped 4 at a time, one spot index per
+//               block column of a bundle, records of 4 int4 per bundle.  Two passes:
+//               private accumulators (rowpriv.cu): every CTA a fixed share of the
+//               active scenarios' work, plain adds in turn, consecutive slots per
+//               scenario; or the ring of path 1 over bundles, with shared atomics.
+//               Sums in float32 or exact 64-bit fixed point (acc64).
+//   With queues (paths 1, 2 and the ring of path 3) the CTA that finishes last
+//   compacts the slots of every scenario into an ordered list, sums the objective
+//   per scenario and resets the queues; with private accumulators it sums the
+//   objective only.
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -84,19 +88,18 @@ struct DevPlan {
   int* err;                           // device error word (bounded waits that ran out)
   int inject_timeout;                 // testing: 1: the ring's producer issues nothing (waits run out); 2: the
                                       // pass with private accumulators gives no turn (as 1 elsewhere)
-  // path 3 (bundled ring): partial slots hold exact 64-bit fixed-point sums.  A
+  // path 3 with exact sums: partial slots hold 64-bit fixed-point sums.  A
   // pass on scenario s scales every contribution by 2^fexp[s], chosen from the
   // bound |acc_c| <= kbound[2s] max|v_s| (+ kbound[2s+1] with the prescription
   // term) so that no sum can overflow; the reducers scale back by 2^-fexp[s].
-  int acc64;                          // 1: partial slots are int64 fixed point (path 3 with exact sums;
-                                      //    0 on path 3: float32 shared atomics, like paths 0-2)
+  int acc64;                          // 1: partial slots are int64 fixed point (path 3 with exact sums; 0: float32)
   int* fexp;                          // [N] scale exponent of the last scatter pass per scenario
-  int priv;                           // path 3: consumer warps of the pass with private accumulators
-                                      // (rowpriv.cu), 0: the ring with atomics; its accumulators (a divisor
-  int priv_acc, ring_bytes;           // of priv) and its ring's bytes; per scenario {bundles of 32 lanes, of 16, of 8, items}, the first unit
-  const int4* cls;                    // (scenario-major, [N+1]) and each unit's first item
-  const int* uoff;
-  const int* ubeg;
+  // path 3, pass with private accumulators (rowpriv.cu):
+  int priv;                           // its consumer warps; 0: the ring with atomics
+  int priv_acc, ring_bytes;           // its accumulators (a divisor of priv) and its ring's bytes
+  const int4* cls;                    // [N] {bundles of 32 lanes, of 16, of 8, items}
+  const int* uoff;                    // [N+1] first unit of each scenario
+  const int* ubeg;                    // first item of each unit, scenario-major
   const double* kbound;               // [2N] max_c sum_i c_s w_i |a_ic| ||a_i||_1 and max_c sum_i c_s w_i |a_ic| p_i
 };
 

@@ -305,10 +305,11 @@ __global__ void k_cg_init(DevPlan P, Ctl* C, const float* __restrict__ partial,
 // zeros, so the result depends on the column index only, not on n, and a problem
 // in a batched plan of more spots follows its own plan bit for bit.  w and u stay
 // in registers between the two halves; the cluster barriers are hardware barriers.
-// Bound: the chain of latencies (scalars, slots, partials, two cluster barriers,
-// one counter).  The scenario's scalars and slots are loaded together; every CTA
-// sends its part of a sum to the shared memory that reads it, so a barrier is
-// followed by local loads only; the counter that finds the last scenario to finish
+// Bound: the chain of latencies (scalars, slots, partials, two cluster barriers, one
+// counter; a third barrier, which says that every CTA has started, is passed by the
+// way).  The scenario's scalars and slots are loaded together; every CTA sends its part
+// of a sum to the shared memory that reads it, so a barrier is followed by local loads
+// only; the counter that finds the last scenario to finish
 // also adds up how many go on; the scalars that don't wait for delta are divided by
 // a second warp while the first adds delta up; the counters are loaded with the rest.
 // Double additions are slow here (two lanes a cycle), hence block_sum_d's form.  The
